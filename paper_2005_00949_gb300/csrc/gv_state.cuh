@@ -1,19 +1,26 @@
 // gv_state.cuh -- device-resident state of a transport call: the
 // double-buffered per-type track queues (the StackBuffer / stage baskets of
-// GeantV Sec. 2.1.2, as structures of arrays), the generation control block
-// and the tally pointers.
+// GeantV Sec. 2.1.2, as arrays of 16-byte parts), the generation control
+// block and the tally pointers.
 #pragma once
 #include "gv_device.cuh"
 
 namespace gv {
 
-// Structure-of-arrays queue of one particle type.
-template <typename R> struct Queue {
-  double *x, *y, *z;
-  R *u, *v, *w, *E, *nlam;
-  unsigned long long *id;
-  unsigned *ev, *step;
-  int *sf;  // sub-slab | flags << 16
+// Track records.  The queue of one particle type is an array of parts: part p
+// holds 16 bytes of every track, so a warp's consecutive tracks are loaded
+// and stored with one coalesced 16-byte access per part and lane.
+//   FP32 (64 B): {x, y} {z, id} {u, v, w, E} {n_lambda, event, step, sf}
+//   FP64 (84 B): {x, y} {z, id} {u, v} {w, E} {n_lambda, event, step} and sf
+// (sf = sub-slab | flags << 16) in an array of its own.
+// Twelve 4- and 8-byte arrays, as before, took three times the accesses and
+// address computations (see load_track).
+template <typename R> struct TrackLayout {
+  static constexpr int parts = sizeof(R) == 4 ? 4 : 5;
+  static constexpr size_t tail = sizeof(R) == 4 ? 0 : sizeof(int);  // bytes per track past the parts
+  static size_t round256(size_t n) { return (n + 255) / 256 * 256; }
+  static size_t part_bytes(long long cap) { return round256(static_cast<size_t>(cap) * 16); }
+  static size_t queue_bytes(long long cap) { return parts * part_bytes(cap) + round256(static_cast<size_t>(cap) * tail); }
 };
 
 // reciprocal node energies staged in shared memory, padded to 16 bytes
@@ -31,6 +38,11 @@ constexpr int kNClaim = 16;
 struct alignas(128) ClaimSlot {
   unsigned n;
 };
+// Fill counter of one output queue, in a 128-byte line of its own: every
+// warp's append and every block's claim is an atomic on one of these words.
+struct alignas(128) FillSlot {
+  unsigned n;
+};
 
 // An interaction request of the split pipeline: the along-step kernel hands
 // a track that is due a discrete interaction to the interaction kernel
@@ -39,28 +51,31 @@ template <typename R> struct alignas(16) GReq {
   double x, y, z;
   unsigned long long id;
   R E, d0, d1, d2;
-  R u[6];        // u2..u7 of the step
+  R u2, u3;      // the sampler's uniforms of the step's counter block 0
   unsigned ev, kk;
   int sf;        // sub-slab | flags << 16
-  int key;       // type * 3 + process
+  int key;       // request key
 };
+// Request keys: type * 3 + process.  Electrons have two processes, and their
+// third key stands for positrons that stopped and annihilate at rest.
 constexpr int kNReqKey = 9;
+constexpr int kKeyRest = 1 * 3 + 2;
 
 // Generation control block.  The last block of every generation writes the
 // plan of the next one; kernels only read it.
 struct Ctl {
   ClaimSlot claims[kNClaim];
-  unsigned cnt[2][3];        // queue fill per buffer parity and type
+  FillSlot cnt[2][3];        // queue fill per buffer parity and type
+  ClaimSlot claim;           // chunk claim counter of the block claims
   unsigned prim_next;        // primaries handed out so far
   unsigned prim_begin, prim_count;
   unsigned chunk_end[4];     // cumulative chunk counts in claim order: e+, e-, gamma, primaries
-  unsigned claim;            // chunk claim counter
   unsigned blocks_done;
   int K;                     // steps per claimed track this generation
   unsigned chunk_B;          // tracks per block claim this generation
   int status;
   int done;
-  int pad;
+  int book;                  // events are counted live (primaries are still waiting on the in-flight cap)
   unsigned ev_started, ev_done;  // events whose live-track count left / returned to zero
   unsigned max_in_flight;        // refill cap of this call (0: none)
   unsigned emax_bits;            // largest primary energy (FP32 bits), for the automatic cap
@@ -78,7 +93,8 @@ struct Ctl {
 
 template <typename R> struct DevState {
   View<R> view;              // global-memory table pointers and constants
-  Queue<R> q[2][3];
+  unsigned char *qmem;       // track queues [parity][type], see TrackLayout
+  unsigned long long q_bytes, q_part;  // bytes of one queue and of one of its parts
   unsigned long long capacity;
   Ctl *ctl;
   const gv_primary *prim;
@@ -104,6 +120,7 @@ template <typename R> struct DevState {
   unsigned xs_bytes, zb_bytes;  // staged into shared memory
   unsigned smem_req_off;        // start of the basketizer's request records
   unsigned smax_off, smax_bytes; // the integral approach's bound, staged into shared memory
+  unsigned thick_off;            // sub-slab thicknesses, staged into shared memory
   unsigned smem_lk_off;          // the block's secondary stack (local_stack)
   int local_stack;
   int grid, adaptive_chunk;  // blocks of the step kernel; spread small populations over all of them

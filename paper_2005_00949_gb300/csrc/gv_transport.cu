@@ -34,10 +34,6 @@
 namespace gv {
 
 // ------------------------------------------------------------------ sinks
-struct BlockCnt {
-  unsigned long long c[16];
-};
-
 // Scoring (SteppingActions, Sec. 3.8.1).  A lane keeps one pending
 // (event, sub-slab) deposit: consecutive deposits of its track to the same sub-slab merge with a
 // compensated (Kahan) sum in R; a deposit to another sub-slab flushes the
@@ -112,12 +108,6 @@ template <typename R> __device__ __forceinline__ void warp_flush(const DevState<
   p.key = kNoKey;
 }
 
-template <typename R, bool EXT = true>
-__device__ __forceinline__ void count(const DevState<R> *S, BlockCnt *bc, unsigned ev, int c, unsigned long long n = 1) {
-  atomicAdd(&bc->c[c], n);
-  if (EXT && S->evcnt) atomicAdd(&S->evcnt[static_cast<size_t>(ev) * GV_NCOUNT + c], n);
-}
-
 template <typename R> struct Trk {
   double x, y, z;
   R u, v, w, E, nlam;
@@ -127,6 +117,14 @@ template <typename R> struct Trk {
 };
 
 __device__ __forceinline__ void set_status(Ctl *ctl, int code) { atomicCAS(&ctl->status, 0, code); }
+
+// The key of a track's random stream and one counter block of step k.
+template <typename R>
+__device__ __forceinline__ uint4 track_draw(const DevState<R> *S, unsigned long long id, unsigned ev, uint32_t k,
+                                            uint32_t block) {
+  return philox4x32_10(make_uint4(static_cast<uint32_t>(id), static_cast<uint32_t>(id >> 32), k, block),
+                       S->seed_lo ^ (ev + S->ev_base), S->seed_hi);
+}
 
 // Integral approach at the post-step point: the process whose cumulative
 // post-step cross section first exceeds `target` (u Sigma_max), or -1 (no
@@ -148,153 +146,184 @@ template <typename R> __device__ __noinline__ int integral_choice(const View<R> 
   return -1;
 }
 
-// ------------------------------------------------------------------ one step
-// PreStep .. process choice of one step.  Returns 1 if the track is still
-// alive; then proc >= 0 names the discrete process due at the post-step
-// point and u[] holds the step's eight uniforms for its final state.
-// Secondaries made so far go to `kids`; kk is the step index whose counter
-// blocks derive the children's ids.
-// FIELD: compiled with the magnetic-field propagation (a field-free kernel
-// keeps its registers for the rest of the step).  OPTS: compiled with the
-// optional processes (multiple scattering, the integral approach); the plain
-// kernel leaves their code out.
-template <typename R, bool FIELD, bool OPTS, bool EXT>
-__device__ int step_track(const View<R> &V, const DevState<R> *S, Trk<R> &t, Kids<R> &kids, uint32_t &kk,
-                          BlockCnt *bc, int &proc_out, R *u, int &lim_out, Pending<R> *pd) {
-  kids.n = 0;
-  proc_out = -1;
-  lim_out = -1;
-  const uint32_t k = t.step;
-  kk = k;
-  const uint32_t key0 = S->seed_lo ^ (t.ev + S->ev_base), key1 = S->seed_hi;
-  const uint32_t idlo = static_cast<uint32_t>(t.id), idhi = static_cast<uint32_t>(t.id >> 32);
-  // counter block 0 is drawn only when the step needs it: a new n_lambda, or
-  // a physics-limited step (process choice and alias uniforms)
-  uint4 r0 = make_uint4(0u, 0u, 0u, 0u);
-  bool have_r0 = false;
-  const R tcut = V.rc.tcut;
-  if (t.E < tcut) {  // PreStep: tracking cut
-    deposit<R, EXT>(V, S, t.ev, t.sub, t.x, t.y, t.E, pd);
-    if (t.type == 2) {
-      const uint4 r1 = philox4x32_10(make_uint4(idlo, idhi, k, 1u), key0, key1);
-      at_rest(kids, u24<R>(r1.z), u24<R>(r1.w));
-      count<R, EXT>(S, bc, t.ev, GV_C_ANNIH);
-    }
-    return 0;
-  }
-  const int mat = V.smat[t.sub];
-  // ComputeIntLen
-  if (t.nlam <= R(0)) {
-    r0 = philox4x32_10(make_uint4(idlo, idhi, k, 0u), key0, key1);
-    have_r0 = true;
-    t.nlam = -m_log(u24<R>(r0.x));
-  }
-  int gi;  // the pre-step energy's grid position serves the lookup and the loss
+// ------------------------------------------------------------------ a run of steps
+// How a track's run of along-steps ended.
+constexpr int kRunOn = 0;    // its budget is used, or a new n_lambda is due: it goes on in the next round
+constexpr int kRunPhys = 1;  // a physics-limited step: the process choice is due
+constexpr int kRunEnd = 2;   // it ended: below the tracking cut, or out of the box
+constexpr int kRunRest = 3;  // a positron stopped: it annihilates at rest
+constexpr int kNoteEpEsc = 1, kNoteUnscat = 2;  // an escaped positron, an unscattered primary
+
+// What a run leaves for the process choice and the step counters.
+template <typename R> struct Run {
+  R sig0, sig1, sig2, Smax;  // cross sections of the last step
+  unsigned n_st, n_geom, n_iter;
+  int note;
+};
+
+// A track left the box (or there is nothing left to stop it).
+template <typename R, bool EXT>
+__device__ __forceinline__ void escape(const View<R> &V, const DevState<R> *S, const Trk<R> &t, int plane, Run<R> &r) {
+  atomicAdd(&S->escape[t.ev], f2d(t.E));
+  if (t.type == 2) r.note |= kNoteEpEsc;
+  if ((t.flags & kFlagPrimary) && !(t.flags & kFlagInteracted) && plane == V.geo.nsub) r.note |= kNoteUnscat;
+}
+
+// Photons: PreStep to the end of a run of at most `budget` steps, every one
+// but the last limited by a boundary.  The energy, and with it the grid
+// position, is the same for the whole run; every step after the first starts
+// on the plane of its sub-slab (distance<ENTERED>), and z is needed only
+// where the run ends, so a step costs the FP64 pipe its two lateral
+// additions instead of three additions, a difference and a conversion.
+template <typename R, bool EXT>
+__device__ __forceinline__ int photon_run(const View<R> &V, const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r) {
+  int gi;
   R gf;
   grid_pos(V, t.E, gi, gf);
-  const V4<R> s4 = lookup_at(V, mat, t.type, gi, gf);
-  const R sig0 = s4.x, sig1 = s4.y, sig2 = (t.type == 1) ? R(0) : s4.z;
-  const R Sig = sig0 + sig1 + sig2;
   const R INF = r_inf<R>();
-  const bool charged = t.type != 0;
-  // integral approach: the step is drawn with the bound Sigma_max(E) of the
-  // cross sections the track can reach; the interaction is accepted at the
-  // post-step point
-  const bool integral = OPTS && charged && (V.cut.mask & GV_P_INTEGRAL);
-  R Smax = Sig;
-  if (integral) {
-    const R *m = V.smax + (mat * 2 + t.type - 1) * kGridN;
-    Smax = m[gi] + gf * (m[gi + 1] - m[gi]);
+  for (int m = 0; m < budget; ++m) {
+    ++r.n_iter;
+    const V4<R> s4 = lookup_at(V, V.smat[t.sub], 0, gi, gf);  // ComputeIntLen
+    r.sig0 = s4.x;
+    r.sig1 = s4.y;
+    r.sig2 = s4.z;
+    const R Sig = r.sig0 + r.sig1 + r.sig2;
+    const R s_phys = Sig > R(0) ? q_div(t.nlam, Sig) : INF;
+    int next, plane;  // GeomQuery
+    const R s_geom = m == 0 ? distance(V, t.x, t.y, t.z, t.u, t.v, t.w, t.sub, next, plane)
+                            : distance<R, true>(V, t.x, t.y, t.z, t.u, t.v, t.w, t.sub, next, plane);
+    R s = INF < s_geom ? INF : s_geom;
+    s = s_phys < s ? s_phys : s;
+    const bool geom = s_geom == s;
+    if (!(s < INF)) {
+      escape<R, EXT>(V, S, t, -1, r);
+      return kRunEnd;
+    }
+    t.x += f2d(s * t.u);
+    t.y += f2d(s * t.v);
+    ++t.step;
+    ++r.n_st;
+    if (!geom) {  // physics (a photon has no other limit)
+      t.z += f2d(s * t.w);
+      t.nlam = R(0);
+      return kRunPhys;
+    }
+    ++r.n_geom;
+    if (Sig > R(0)) t.nlam = t.nlam - s * Sig;
+    if (next < 0) {
+      escape<R, EXT>(V, S, t, plane, r);
+      return kRunEnd;
+    }
+    t.z = V.zb[plane];
+    t.sub = next;
+    if (t.nlam <= R(0)) break;
   }
-  const R s_phys = Smax > R(0) ? q_div(t.nlam, Smax) : INF;
-  R s_cont = INF, Rr = R(0);
-  if (charged) {
-    Rr = range_of(s4, t.type);
+  return kRunOn;
+}
+
+// Electrons and positrons: a run of at most `budget` steps, each limited by
+// a boundary, by the continuous loss (or the field) or, the last one, by
+// physics.
+template <typename R, bool FIELD, bool OPTS, bool EXT>
+__device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r,
+                                           Pending<R> *pd) {
+  const R INF = r_inf<R>();
+  for (int m = 0; m < budget; ++m) {
+    ++r.n_iter;
+    const int mat = V.smat[t.sub];
+    // ComputeIntLen; the pre-step energy's grid position serves the lookup and the loss
+    int gi;
+    R gf;
+    grid_pos(V, t.E, gi, gf);
+    const V4<R> s4 = lookup_at(V, mat, t.type, gi, gf);
+    r.sig0 = s4.x;
+    r.sig1 = s4.y;
+    r.sig2 = (t.type == 1) ? R(0) : s4.z;
+    const R Sig = r.sig0 + r.sig1 + r.sig2;
+    // integral approach: the step is drawn with the bound Sigma_max(E) of the
+    // cross sections the track can reach; the interaction is accepted at the
+    // post-step point
+    R Smax = Sig;
+    if (OPTS && (V.cut.mask & GV_P_INTEGRAL)) {
+      const R *mx = V.smax + (mat * 2 + t.type - 1) * kGridN;
+      Smax = mx[gi] + gf * (mx[gi + 1] - mx[gi]);
+    }
+    r.Smax = Smax;
+    const R s_phys = Smax > R(0) ? q_div(t.nlam, Smax) : INF;
+    const R Rr = range_of(s4, t.type);
     const R a = static_cast<R>(kAlphaR) * Rr, b = Rr < static_cast<R>(kRhoF) ? Rr : static_cast<R>(kRhoF);
-    s_cont = a > b ? a : b;
+    R s_cont = a > b ? a : b;
     if (FIELD && V.rc.field_k != R(0)) {  // the field's step limit acts like the continuous one
       const R sf = field_limit(V, t.type, t.E, t.u, t.v, t.w);
       s_cont = sf < s_cont ? sf : s_cont;
     }
-  }
-  // GeomQuery
-  int next, plane;
-  const R s_geom = distance(V, t.x, t.y, t.z, t.u, t.v, t.w, t.sub, next, plane);
-  R s = s_cont < s_geom ? s_cont : s_geom;
-  s = s_phys < s ? s_phys : s;
-  const int lim = (s_geom == s) ? 0 : (s_phys == s ? 1 : 2);
-  lim_out = lim;
-  if (!(s < INF)) {
-    atomicAdd(&S->escape[t.ev], f2d(t.E));
-    if (t.type == 2) count<R, EXT>(S, bc, t.ev, GV_C_EP_ESC);
-    return 0;
-  }
-  // Propagation: FP64 positions, advanced by displacements s d formed in R
-  // (s and d are R already; an FP32 displacement is widened exactly on the
-  // integer ALU, leaving the FP64 pipe one addition per coordinate; in FP64
-  // mode this is one fused multiply-add)
-  double mx = 0.0, my = 0.0;  // step midpoint: only cell scoring reads it
-  if (FIELD && charged && V.rc.field_k != R(0)) {  // the helix of the pre-step momentum
-    const R d0[3] = {t.u, t.v, t.w};
-    R dp[3], nd[3];
-    if (EXT && S->cell) {
-      helix(V, t.type, t.E, R(0.5) * s, d0, dp, nd);
-      mx = t.x + f2d(dp[0]);
-      my = t.y + f2d(dp[1]);
+    // GeomQuery
+    int next, plane;
+    const R s_geom = distance(V, t.x, t.y, t.z, t.u, t.v, t.w, t.sub, next, plane);
+    R s = s_cont < s_geom ? s_cont : s_geom;
+    s = s_phys < s ? s_phys : s;
+    const int lim = (s_geom == s) ? 0 : (s_phys == s ? 1 : 2);
+    if (!(s < INF)) {
+      escape<R, EXT>(V, S, t, -1, r);
+      return kRunEnd;
     }
-    helix(V, t.type, t.E, s, d0, dp, nd);
-    t.x += f2d(dp[0]);
-    t.y += f2d(dp[1]);
-    t.z += f2d(dp[2]);
-    if (lim == 0) {  // the crossed plane, chosen with the pre-step direction
-      if (plane >= 0) t.z = V.zb[plane];
-      else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
-      else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
+    // Propagation: FP64 positions, advanced by displacements s d formed in R
+    // (s and d are R already; an FP32 displacement is widened exactly on the
+    // integer ALU, leaving the FP64 pipe one addition per coordinate; in FP64
+    // mode this is one fused multiply-add)
+    double mx = 0.0, my = 0.0;  // step midpoint: only cell scoring reads it
+    if (FIELD && V.rc.field_k != R(0)) {  // the helix of the pre-step momentum
+      const R d0[3] = {t.u, t.v, t.w};
+      R dp[3], nd[3];
+      if (EXT && S->cell) {
+        helix(V, t.type, t.E, R(0.5) * s, d0, dp, nd);
+        mx = t.x + f2d(dp[0]);
+        my = t.y + f2d(dp[1]);
+      }
+      helix(V, t.type, t.E, s, d0, dp, nd);
+      t.x += f2d(dp[0]);
+      t.y += f2d(dp[1]);
+      t.z += f2d(dp[2]);
+      if (lim == 0) {  // the crossed plane, chosen with the pre-step direction
+        if (plane >= 0) t.z = V.zb[plane];
+        else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
+        else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
+      }
+      t.u = nd[0];
+      t.v = nd[1];
+      t.w = nd[2];
+    } else {
+      if (EXT && S->cell) {
+        mx = t.x + f2d(R(0.5) * s * t.u);
+        my = t.y + f2d(R(0.5) * s * t.v);
+      }
+      t.x += f2d(s * t.u);
+      t.y += f2d(s * t.v);
+      t.z += f2d(s * t.w);
+      if (lim == 0) {
+        if (plane >= 0) t.z = V.zb[plane];
+        else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
+        else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
+      }
     }
-    t.u = nd[0];
-    t.v = nd[1];
-    t.w = nd[2];
-  } else {
-    if (EXT && S->cell) {
-      mx = t.x + f2d(R(0.5) * s * t.u);
-      my = t.y + f2d(R(0.5) * s * t.v);
-    }
-    t.x += f2d(s * t.u);
-    t.y += f2d(s * t.v);
-    t.z += f2d(s * t.w);
-    if (lim == 0) {
-      if (plane >= 0) t.z = V.zb[plane];
-      else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
-      else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
-    }
-  }
-  if (Smax > R(0)) t.nlam = (lim == 1) ? R(0) : t.nlam - s * Smax;
-  t.step = k + 1;
-  // the block's step counters are summed per warp by the caller; only the
-  // optional per-event rows are booked here
-  if (EXT && S->evcnt) {
-    atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_STEPS], 1ull);
-    atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_STEPS_G + t.type], 1ull);
-  }
-  const int pre_sub = t.sub;
-  const R E_pre = t.E;
-  // AlongStepAction
-  if (charged) {
+    if (Smax > R(0)) t.nlam = (lim == 1) ? R(0) : t.nlam - s * Smax;
+    const uint32_t k = t.step;
+    t.step = k + 1;
+    ++r.n_st;
+    r.n_geom += lim == 0 ? 1u : 0u;
+    const int pre_sub = t.sub;
+    const R E_pre = t.E;
+    // AlongStepAction
     const R Ep = eloss_at(V, mat, t.type, t.E, gi, gf, s, Rr);
     deposit<R, EXT>(V, S, t.ev, pre_sub, mx, my, t.E - Ep, pd);
     t.E = Ep;
-    if (t.E < tcut) {
+    if (t.E < V.rc.tcut) {
       deposit<R, EXT>(V, S, t.ev, pre_sub, t.x, t.y, t.E, pd);
-      if (t.type == 2) {
-        const uint4 r1 = philox4x32_10(make_uint4(idlo, idhi, k, 1u), key0, key1);
-        at_rest(kids, u24<R>(r1.z), u24<R>(r1.w));
-        count<R, EXT>(S, bc, t.ev, GV_C_ANNIH);
-      }
-      return 0;
+      return t.type == 2 ? kRunRest : kRunEnd;
     }
     // multiple scattering of a track that stays in the box (counter block 2)
     if (OPTS && (V.cut.mask & GV_P_MSC) && !(lim == 0 && next < 0)) {
-      const uint4 r2 = philox4x32_10(make_uint4(idlo, idhi, k, 2u), key0, key1);
+      const uint4 r2 = track_draw(S, t.id, t.ev, k, 2u);
       const R um[4] = {u24<R>(r2.x), u24<R>(r2.y), u24<R>(r2.z), u24<R>(r2.w)};
       R dm[3] = {t.u, t.v, t.w};
       msc_step(V, pre_sub, E_pre, t.E, s, dm, t.x, t.y, t.z, um);
@@ -302,103 +331,261 @@ __device__ int step_track(const View<R> &V, const DevState<R> *S, Trk<R> &t, Kid
       t.v = dm[1];
       t.w = dm[2];
     }
-  }
-  if (lim == 0) {
-    if (next < 0) {
-      atomicAdd(&S->escape[t.ev], f2d(t.E));
-      if (t.type == 2) count<R, EXT>(S, bc, t.ev, GV_C_EP_ESC);
-      if ((t.flags & kFlagPrimary) && !(t.flags & kFlagInteracted) && plane == V.geo.nsub)
-        count<R, EXT>(S, bc, t.ev, GV_C_UNSCAT);
-      return 0;
+    if (lim == 0) {
+      if (next < 0) {
+        escape<R, EXT>(V, S, t, plane, r);
+        return kRunEnd;
+      }
+      t.sub = next;
+    } else if (lim == 1) {
+      return kRunPhys;
     }
-    t.sub = next;
-    return 1;
+    if (t.nlam <= R(0)) break;
   }
-  if (lim != 1) return 1;
-  // PostStepActions: process choice, then the final state
-  if (!have_r0) r0 = philox4x32_10(make_uint4(idlo, idhi, k, 0u), key0, key1);
-  int proc = -1;
-  if (integral) {  // post-step cross sections; above their sum: no interaction
-    proc = integral_choice(V, mat, t.type, t.E, u24<R>(r0.y) * Smax);
+  return kRunOn;
+}
+
+// One round of a track: PreStep, a new n_lambda where one is due, a run of
+// along-steps, and the process choice after a physics-limited one.  Returns
+// the request key of the final state now due (type * 3 + process, or
+// kKeyRest), or -1; kk is the step whose counter blocks its final state
+// draws from, u2 and u3 the words of block 0 it samples with.  `alive` falls
+// when the track ended or handed itself to an at-rest annihilation.
+//
+// The random numbers are drawn here once per round, outside the loop over
+// steps: a step that leaves a track without n_lambda (an interaction is the
+// rule, a rounding in n_lambda - s Sigma the exception) ends its run, so
+// that its warp draws for all of its tracks together; the second block of an
+// interaction is drawn by the lane that runs its final state.  Inside the
+// loop every draw ran for whichever few lanes of the warp were due it.
+template <typename R, bool FIELD, bool OPTS, bool EXT>
+__device__ __forceinline__ int run_round(const View<R> &V, const DevState<R> *S, Trk<R> &t, bool &alive, int budget_g,
+                                         int budget, uint32_t &kk, R &u2, R &u3, Run<R> &r, Pending<R> *pd) {
+  r.n_st = r.n_geom = r.n_iter = 0;
+  r.note = 0;
+  kk = 0;
+  if (!alive) return -1;
+  int end;
+  if (t.E < V.rc.tcut) {  // PreStep: tracking cut
+    r.n_iter = 1;
+    kk = t.step;
+    deposit<R, EXT>(V, S, t.ev, t.sub, t.x, t.y, t.E, pd);
+    end = t.type == 2 ? kRunRest : kRunEnd;
   } else {
-    const R target = u24<R>(r0.y) * Sig;
-    R cum = sig0;
+    if (t.nlam <= R(0)) t.nlam = -m_log(u24<R>(track_draw(S, t.id, t.ev, t.step, 0u).x));
+    end = t.type == 0 ? photon_run<R, EXT>(V, S, t, budget_g, r)
+                      : charged_run<R, FIELD, OPTS, EXT>(V, S, t, budget, r, pd);
+    kk = t.step - 1u;
+  }
+  if (EXT && S->evcnt && (r.n_st || r.note)) {  // the optional per-event rows
+    unsigned long long *row = &S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT];
+    atomicAdd(&row[GV_C_STEPS], static_cast<unsigned long long>(r.n_st));
+    atomicAdd(&row[GV_C_STEPS_G + t.type], static_cast<unsigned long long>(r.n_st));
+    if (r.note & kNoteEpEsc) atomicAdd(&row[GV_C_EP_ESC], 1ull);
+    if (r.note & kNoteUnscat) atomicAdd(&row[GV_C_UNSCAT], 1ull);
+  }
+  // NaN energy, or a non-finite z (tested on its exponent bits: an FP64
+  // comparison would take the FP64 pipe)
+  if (!(t.E == t.E) || (__double2hiint(t.z) & 0x7ff00000) == 0x7ff00000) {
+    set_status(S->ctl, GV_ERR_NUMERIC);
+    alive = false;
+    return -1;
+  }
+  if (end == kRunEnd || end == kRunRest) {
+    alive = false;
+    return end == kRunRest ? kKeyRest : -1;
+  }
+  if (end == kRunOn) return -1;
+  // PostStepActions: process choice
+  const uint4 r0 = track_draw(S, t.id, t.ev, kk, 0u);
+  int proc = -1;
+  if (OPTS && t.type != 0 && (V.cut.mask & GV_P_INTEGRAL)) {  // post-step cross sections; above their sum: no interaction
+    proc = integral_choice(V, V.smat[t.sub], t.type, t.E, u24<R>(r0.y) * r.Smax);
+  } else {
+    const R target = u24<R>(r0.y) * (r.sig0 + r.sig1 + r.sig2);
+    R cum = r.sig0;
     if (target < cum) proc = 0;
     else {
-      cum += sig1;
+      cum += r.sig1;
       if (target < cum) proc = 1;
       else {
-        cum += sig2;
+        cum += r.sig2;
         if (target < cum) proc = 2;
       }
     }
-    if (proc < 0) proc = sig2 > R(0) ? 2 : (sig1 > R(0) ? 1 : (sig0 > R(0) ? 0 : -1));
+    if (proc < 0) proc = r.sig2 > R(0) ? 2 : (r.sig1 > R(0) ? 1 : (r.sig0 > R(0) ? 0 : -1));
   }
   t.nlam = R(-1);
-  if (proc < 0) return 1;
-  const uint4 r1 = philox4x32_10(make_uint4(idlo, idhi, k, 1u), key0, key1);
-  u[0] = u24<R>(r0.x); u[1] = u24<R>(r0.y); u[2] = u24<R>(r0.z); u[3] = u24<R>(r0.w);
-  u[4] = u24<R>(r1.x); u[5] = u24<R>(r1.y); u[6] = u24<R>(r1.z); u[7] = u24<R>(r1.w);
-  proc_out = proc;
-  return 1;
+  u2 = u24<R>(r0.z);
+  u3 = u24<R>(r0.w);
+  return proc < 0 ? -1 : t.type * 3 + proc;
 }
 
-// PostStepActions of a track whose step ended in process `proc`: the final
-// state, the local deposit and the counters.  Returns 1 if the particle
-// survives, 0 if it ended, -1 if the process was kinematically closed at the
-// post-step energy (nothing changes).
+// PostStepActions of the request `key`: the final state and its local
+// deposit.  Returns 1 if the particle survives, 0 if it ended, -1 if the
+// process was kinematically closed at the post-step energy (nothing
+// changes).  np, na: pairs and annihilations made.
 template <typename R, bool OPTS = true, bool EXT = true>
-__device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *S, BlockCnt *bc, int type, int proc,
-                                           R &E, R d[3], const R *u, Kids<R> &kids, unsigned ev, int sub,
-                                           double x, double y, unsigned long long id, uint32_t kk,
+__device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *S, int key, R &E, R d[3], R u2, R u3,
+                                           Kids<R> &kids, unsigned ev, int sub, double x, double y,
+                                           unsigned long long id, uint32_t kk, int &np, int &na,
                                            Pending<R> *pd = nullptr) {
-  R local;
-  int np = 0, na = 0;
-  const RngKey g = {static_cast<uint32_t>(id), static_cast<uint32_t>(id >> 32), kk, S->seed_lo ^ (ev + S->ev_base),
-                    S->seed_hi};
-  const int r = interact<R, OPTS>(V, type, proc, E, d, u, g, kids, local, np, na);
-  if (r < 0) return -1;
-  if (np) count<R, EXT>(S, bc, ev, GV_C_PAIR, np);
-  if (na) count<R, EXT>(S, bc, ev, GV_C_ANNIH, na);
-  deposit<R, EXT>(V, S, ev, sub, x, y, local, pd);
+  const uint4 r1 = track_draw(S, id, ev, kk, 1u);
+  const R u[8] = {R(0), R(0), u2, u3, u24<R>(r1.x), u24<R>(r1.y), u24<R>(r1.z), u24<R>(r1.w)};
+  int r = 0;
+  if (key == kKeyRest) {
+    at_rest(kids, u[6], u[7]);
+    na = 1;
+  } else {
+    const int type = key / 3;
+    R local;
+    const RngKey g = {static_cast<uint32_t>(id), static_cast<uint32_t>(id >> 32), kk, S->seed_lo ^ (ev + S->ev_base),
+                      S->seed_hi};
+    r = interact<R, OPTS>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na);
+    if (r < 0) return -1;
+    deposit<R, EXT>(V, S, ev, sub, x, y, local, pd);
+  }
+  if (EXT && S->evcnt) {
+    unsigned long long *row = &S->evcnt[static_cast<size_t>(ev) * GV_NCOUNT];
+    if (np) atomicAdd(&row[GV_C_PAIR], static_cast<unsigned long long>(np));
+    if (na) atomicAdd(&row[GV_C_ANNIH], static_cast<unsigned long long>(na));
+  }
   return r;
 }
 
-// ------------------------------------------------------------------ queues
-// Warp-aggregated append: each lane contributes c_q records of type q; one
-// atomic per warp and type reserves the slots.  Must be called by all 32
-// lanes of a converged warp.
-__device__ __forceinline__ unsigned warp_reserve(unsigned *counter, unsigned c, unsigned &total) {
-  const int lane = threadIdx.x & 31;
-  unsigned incl = c;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+// ------------------------------------------------------------------ counters
+// Counters of one warp: 16 words of shared memory that only this warp
+// writes, lane c to counter c, so that booking takes no atomic (64-bit
+// shared-memory atomics are compare-and-swap loops).
+using WarpCnt = unsigned long long[16];
+
+__device__ __forceinline__ void wcnt_add(unsigned long long *row, int c, unsigned v) {
+  if ((threadIdx.x & 31) == static_cast<unsigned>(c)) row[c] += v;
+}
+
+// The step counters of one round.  All 32 lanes of a converged warp.
+template <typename R>
+__device__ __forceinline__ void count_round(unsigned long long *row, const Run<R> &r, int type, bool chose) {
+  // steps, boundary-limited steps (at most 64 per lane) and process choices in one sum
+  const unsigned sum = __reduce_add_sync(0xffffffffu, r.n_st | (r.n_geom << 12) | (chose ? 1u << 24 : 0u));
+  const unsigned it = __reduce_max_sync(0xffffffffu, r.n_iter);
+  const unsigned st = sum & 0xfffu;
+  const unsigned mg = __ballot_sync(0xffffffffu, r.n_st && type == 0);
+  const unsigned me = __ballot_sync(0xffffffffu, r.n_st && type == 1);
+  const unsigned mp = __ballot_sync(0xffffffffu, r.n_st && type == 2);
+  unsigned wg = st, we = st;
+  if ((mg != 0) + (me != 0) + (mp != 0) > 1) {  // mixed types: primaries, or the block's stack
+    wg = __reduce_add_sync(0xffffffffu, type == 0 ? r.n_st : 0u);
+    we = __reduce_add_sync(0xffffffffu, type == 1 ? r.n_st : 0u);
+  } else {
+    wg = mg ? st : 0u;
+    we = me ? st : 0u;
   }
-  total = __shfl_sync(0xffffffffu, incl, 31);
-  unsigned base = 0;
-  if (lane == 31 && total) base = atomicAdd(counter, total);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  return base + incl - c;
+  const int lane = threadIdx.x & 31;
+  unsigned v = 0;
+  if (lane == GV_C_STEPS) v = st;
+  if (lane == GV_C_STEPS_G) v = wg;
+  if (lane == GV_C_STEPS_EM) v = we;
+  if (lane == GV_C_STEPS_EP) v = st - wg - we;
+  if (lane == GV_C_GEOM) v = (sum >> 12) & 0xfffu;
+  if (lane == GV_C_DISCRETE) v = sum >> 24;
+  if (lane == GV_C_LANE_SLOTS) v = 32u * it;  // idle-lane fraction
+  if (v) row[lane] += v;
+  if (__any_sync(0xffffffffu, r.note)) {
+    const unsigned esc = __popc(__ballot_sync(0xffffffffu, r.note & kNoteEpEsc));
+    const unsigned uns = __popc(__ballot_sync(0xffffffffu, r.note & kNoteUnscat));
+    wcnt_add(row, GV_C_EP_ESC, esc);
+    wcnt_add(row, GV_C_UNSCAT, uns);
+  }
+}
+
+// ------------------------------------------------------------------ queues
+__device__ __forceinline__ double i2d(unsigned long long v) { return __longlong_as_double(static_cast<long long>(v)); }
+__device__ __forceinline__ unsigned long long d2i(double v) {
+  return static_cast<unsigned long long>(__double_as_longlong(v));
+}
+
+// One track record read from or written to queue (par, type), see
+// TrackLayout.
+template <typename R>
+__device__ __forceinline__ void load_track(const DevState<R> *S, int par, int type, unsigned slot, Trk<R> &t) {
+  const unsigned char *b = S->qmem + static_cast<unsigned>(par * 3 + type) * S->q_bytes;
+  const unsigned char *p = b + static_cast<unsigned long long>(slot) * 16u;
+  const unsigned long long part = S->q_part;
+  const double2 a = *reinterpret_cast<const double2 *>(p);
+  const double2 c = *reinterpret_cast<const double2 *>(p + part);
+  t.x = a.x; t.y = a.y;
+  t.z = c.x; t.id = d2i(c.y);
+  int sf;
+  if constexpr (sizeof(R) == 4) {
+    const float4 d = *reinterpret_cast<const float4 *>(p + 2 * part);
+    const uint4 e = *reinterpret_cast<const uint4 *>(p + 3 * part);
+    t.u = d.x; t.v = d.y; t.w = d.z; t.E = d.w;
+    t.nlam = __uint_as_float(e.x); t.ev = e.y; t.step = e.z;
+    sf = static_cast<int>(e.w);
+  } else {
+    const double2 d = *reinterpret_cast<const double2 *>(p + 2 * part);
+    const double2 f = *reinterpret_cast<const double2 *>(p + 3 * part);
+    const uint4 e = *reinterpret_cast<const uint4 *>(p + 4 * part);
+    t.u = d.x; t.v = d.y; t.w = f.x; t.E = f.y;
+    t.nlam = __hiloint2double(static_cast<int>(e.y), static_cast<int>(e.x));
+    t.ev = e.z; t.step = e.w;
+    sf = reinterpret_cast<const int *>(b + 5 * part)[slot];
+  }
+  t.sub = sf & 0xffff;
+  t.flags = sf >> 16;
+  t.type = type;
 }
 
 template <typename R>
-__device__ __forceinline__ void store(const Queue<R> &q, unsigned slot, double x, double y, double z, R u, R v, R w,
-                                      R E, R nlam, unsigned long long id, unsigned ev, unsigned step, int sf) {
-  q.x[slot] = x;
-  q.y[slot] = y;
-  q.z[slot] = z;
-  q.u[slot] = u;
-  q.v[slot] = v;
-  q.w[slot] = w;
-  q.E[slot] = E;
-  q.nlam[slot] = nlam;
-  q.id[slot] = id;
-  q.ev[slot] = ev;
-  q.step[slot] = step;
-  q.sf[slot] = sf;
+__device__ __forceinline__ void store_track(const DevState<R> *S, int par, int type, unsigned slot, double x, double y,
+                                            double z, R u, R v, R w, R E, R nlam, unsigned long long id, unsigned ev,
+                                            unsigned step, int sf) {
+  unsigned char *b = S->qmem + static_cast<unsigned>(par * 3 + type) * S->q_bytes;
+  unsigned char *p = b + static_cast<unsigned long long>(slot) * 16u;
+  const unsigned long long part = S->q_part;
+  *reinterpret_cast<double2 *>(p) = make_double2(x, y);
+  *reinterpret_cast<double2 *>(p + part) = make_double2(z, i2d(id));
+  if constexpr (sizeof(R) == 4) {
+    *reinterpret_cast<float4 *>(p + 2 * part) = make_float4(u, v, w, E);
+    *reinterpret_cast<uint4 *>(p + 3 * part) = make_uint4(__float_as_uint(nlam), ev, step, static_cast<unsigned>(sf));
+  } else {
+    *reinterpret_cast<double2 *>(p + 2 * part) = make_double2(u, v);
+    *reinterpret_cast<double2 *>(p + 3 * part) = make_double2(w, E);
+    *reinterpret_cast<uint4 *>(p + 4 * part) =
+        make_uint4(static_cast<unsigned>(__double2loint(nlam)), static_cast<unsigned>(__double2hiint(nlam)), ev, step);
+    reinterpret_cast<int *>(b + 5 * part)[slot] = sf;
+  }
 }
+
+// Warp-aggregated append.  A warp adds its lanes' records type by type to
+// n[], each lane keeping its record's rank within its type, and then
+// reserves the slots of all three types with one atomic instruction (lane q
+// for type q): one round trip to L2, where a reservation per type took up to
+// three in a row.  All 32 lanes of a converged warp.
+struct WarpAppend {
+  unsigned n[3] = {0, 0, 0};
+  __device__ __forceinline__ unsigned add(bool has, int type) {
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
+    unsigned rank = 0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const unsigned m = __ballot_sync(0xffffffffu, has && type == q);
+      if (type == q) rank = n[q] + __popc(m & lt);
+      n[q] += __popc(m);
+    }
+    return rank;
+  }
+  // lane q: the first slot of type q; read with slot()
+  __device__ __forceinline__ unsigned reserve(FillSlot *fill) const {
+    const int lane = threadIdx.x & 31;
+    const unsigned mine = lane == 0 ? n[0] : (lane == 1 ? n[1] : (lane == 2 ? n[2] : 0u));
+    return mine ? atomicAdd(&fill[lane].n, mine) : 0u;
+  }
+  __device__ __forceinline__ static unsigned slot(unsigned base, int type, unsigned rank) {
+    return __shfl_sync(0xffffffffu, base, type) + rank;
+  }
+};
 
 // The parent of a step's secondaries: where they start and whose lineage
 // names them.
@@ -409,104 +596,131 @@ struct Parent {
   int sub;
 };
 
-template <typename R> __device__ __forceinline__ Parent parent_of(const Trk<R> &t) {
-  Parent p;
-  p.x = t.x; p.y = t.y; p.z = t.z;
-  p.id = t.id;
-  p.ev = t.ev;
-  p.sub = t.sub;
-  return p;
-}
-
-// A secondary kept in the block's shared-memory stack (the StackBuffer of
-// Sec. 2.1.2 for one block): its lanes take it up in a later round of the
-// same claim instead of leaving it to the next generation.
-template <typename R> struct LKid {
-  double x, y, z;
-  unsigned long long id;
-  R u, v, w, E;
-  unsigned ev;
-  int sub, type;
-};
-
-// The block's secondary stack: `top` entries (it may run past `cap` while
-// appends overflow to the global queues, and below 0 while empty lanes try
-// to pop; both are only ever read through the bounds below).
+// The block's secondary stack in shared memory (the StackBuffer of Sec.
+// 2.1.2 for one block): its lanes take the secondaries up in a later round of
+// the same claim instead of leaving them to the next generation.  Stored like
+// the queues, in 16-byte parts: {x, y} {z, id} {u, v, w, E} {event, sub,
+// type, -}.  `top` counts the entries: appends take back what overflowed to
+// the global queues, and what empty lanes popped below 0 is brought back to 0
+// before the next appends.
 template <typename R> struct LocalStack {
-  LKid<R> *e;
+  unsigned char *e;
   int *top;
   int cap;
+  static constexpr int kBytes = 48 + 4 * sizeof(R);  // per entry
+  __device__ __forceinline__ void put(int i, const Parent &p, unsigned long long id, const R *d, R E, int type) const {
+    reinterpret_cast<double2 *>(e)[i] = make_double2(p.x, p.y);
+    reinterpret_cast<double2 *>(e + 16 * cap)[i] = make_double2(p.z, i2d(id));
+    reinterpret_cast<uint4 *>(e + 32 * cap)[i] = make_uint4(p.ev, static_cast<unsigned>(p.sub), static_cast<unsigned>(type), 0u);
+    reinterpret_cast<V4<R> *>(e + 48 * cap)[i] = V4<R>{d[0], d[1], d[2], E};
+  }
+  __device__ __forceinline__ void get(int i, Trk<R> &t) const {
+    const double2 a = reinterpret_cast<const double2 *>(e)[i];
+    const double2 c = reinterpret_cast<const double2 *>(e + 16 * cap)[i];
+    const uint4 g = reinterpret_cast<const uint4 *>(e + 32 * cap)[i];
+    const V4<R> d = reinterpret_cast<const V4<R> *>(e + 48 * cap)[i];
+    t.x = a.x; t.y = a.y; t.z = c.x;
+    t.id = d2i(c.y);
+    t.u = d.x; t.v = d.y; t.w = d.z; t.E = d.w;
+    t.nlam = R(-1);
+    t.ev = g.x;
+    t.step = 0;
+    t.sub = static_cast<int>(g.y);
+    t.type = static_cast<int>(g.z);
+    t.flags = 0;
+  }
 };
 
 // PostStepActions: append the step's secondaries to the output queues, or,
 // with a local stack, to the block's stack while it has room.  Called by all
 // 32 lanes of a converged warp (lanes without secondaries pass kids.n == 0).
 template <typename R, bool EXT = true>
-__device__ void push_kids(const DevState<R> *S, int out, const Parent &t, const Kids<R> &kids, uint32_t kk,
-                          BlockCnt *bc, const LocalStack<R> *ls = nullptr) {
-  const unsigned any = __ballot_sync(0xffffffffu, kids.n > 0);
-  if (!any) return;
+__device__ __forceinline__ void push_kids(const DevState<R> *S, int out, const Parent &t, const Kids<R> &kids,
+                                          uint32_t kk, unsigned long long *row, const LocalStack<R> *ls = nullptr) {
+  const unsigned b0 = __ballot_sync(0xffffffffu, kids.n > 0);
+  if (!b0) return;
+  const int lane = threadIdx.x & 31;
   uint32_t w[6] = {0, 0, 0, 0, 0, 0};
   if (kids.n > 0) {
-    const uint32_t key0 = S->seed_lo ^ (t.ev + S->ev_base);
-    const uint4 a = philox4x32_10(make_uint4(static_cast<uint32_t>(t.id), static_cast<uint32_t>(t.id >> 32), kk, kTagId),
-                                  key0, S->seed_hi);
+    const uint4 a = track_draw(S, t.id, t.ev, kk, kTagId);
     w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
     if (kids.n > 2) {
-      const uint4 b = philox4x32_10(
-          make_uint4(static_cast<uint32_t>(t.id), static_cast<uint32_t>(t.id >> 32), kk, kTagId + 1u), key0, S->seed_hi);
+      const uint4 b = track_draw(S, t.id, t.ev, kk, kTagId + 1u);
       w[4] = b.x; w[5] = b.y;
     }
   }
+  const unsigned b1 = __ballot_sync(0xffffffffu, kids.n > 1);
+  const unsigned b2 = __ballot_sync(0xffffffffu, kids.n > 2);
   // the block's stack first, while it has room (the ids above keep each
   // kid's index in the list, so where it goes changes no result)
-  unsigned local = 0;  // bit j: kid j went to the block's stack
+  int room = 0;  // the lane's first `room` kids go to the block's stack
   if (ls) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (j >= kids.n) continue;
-      const int slot = atomicAdd(ls->top, 1);
-      if (slot < 0 || slot >= ls->cap) continue;
-      LKid<R> &e = ls->e[slot];
-      e.x = t.x; e.y = t.y; e.z = t.z;
-      e.id = static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32);
-      e.u = kids.d[j][0]; e.v = kids.d[j][1]; e.w = kids.d[j][2];
-      e.E = kids.E[j];
-      e.ev = t.ev;
-      e.sub = t.sub;
-      e.type = kids.type[j];
-      atomicAdd(&bc->c[GV_C_TRK_G + kids.type[j]], 1ull);
-      if (EXT && S->evcnt) atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
-      local |= 1u << j;
+    int base = 0;
+    if (lane == 0) {
+      const int tot = __popc(b0) + __popc(b1) + __popc(b2);
+      base = atomicAdd(ls->top, tot);
+      const int over = min(tot, base + tot - ls->cap);
+      if (over > 0) atomicSub(ls->top, over);
     }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const unsigned lt = (1u << lane) - 1u;
+    base += __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt);
+    room = max(0, min(ls->cap - base, kids.n));
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (j < room)
+        ls->put(base + j, t, static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
+                kids.d[j], kids.E[j], kids.type[j]);
+  }
+  WarpAppend ap, all;
+  unsigned rank[3] = {0, 0, 0};
+  const unsigned bj[3] = {b0, b1, b2};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (!bj[j]) continue;
+    if (ls) all.add(j < kids.n, kids.type[j]);
+    rank[j] = ap.add(j < kids.n && j >= room, kids.type[j]);
   }
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    unsigned c = 0;
+  for (int q = 0; q < 3; ++q) wcnt_add(row, GV_C_TRK_G + q, ls ? all.n[q] : ap.n[q]);
+  if (EXT && S->evcnt) {
 #pragma unroll
-    for (int j = 0; j < 3; ++j) c += (j < kids.n && kids.type[j] == q && !(local >> j & 1u)) ? 1u : 0u;
-    if (!__ballot_sync(0xffffffffu, c > 0)) continue;
-    unsigned total;
-    unsigned slot = warp_reserve(&S->ctl->cnt[out][q], c, total);
-    if ((threadIdx.x & 31) == 0 && total) atomicAdd(&bc->c[GV_C_TRK_G + q], static_cast<unsigned long long>(total));
-    if (c == 0) continue;
-    if (slot + c > S->capacity) {
+    for (int j = 0; j < 3; ++j)
+      if (j < kids.n) atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
+  }
+  if (!(ap.n[0] | ap.n[1] | ap.n[2])) return;
+  const unsigned base = ap.reserve(S->ctl->cnt[out]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (!bj[j]) continue;
+    const bool has = j < kids.n && j >= room;
+    const unsigned slot = WarpAppend::slot(base, has ? kids.type[j] : 0, rank[j]);
+    if (!has) continue;
+    if (slot >= S->capacity) {
       set_status(S->ctl, GV_ERR_STACK_FULL);
       continue;
     }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (!(j < kids.n && kids.type[j] == q) || (local >> j & 1u)) continue;
-      const unsigned long long id = static_cast<unsigned long long>(w[2 * j]) |
-                                    (static_cast<unsigned long long>(w[2 * j + 1]) << 32);
-      store(S->q[out][q], slot, t.x, t.y, t.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j], R(-1), id, t.ev,
-            0u, t.sub);
-      if (EXT && S->evcnt) atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_TRK_G + q], 1ull);
-      ++slot;
-    }
+    store_track<R>(S, out, kids.type[j], slot, t.x, t.y, t.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j],
+                   R(-1), static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
+                   t.ev, 0u, t.sub);
   }
-  // the event's live-track count grows before the parent's own end is booked
-  if (kids.n > 0) atomicAdd(&S->evlive[t.ev], static_cast<unsigned>(kids.n));
+}
+
+// Survivors: one record per lane (has: whether it has one).  All 32 lanes of
+// a converged warp.
+template <typename R>
+__device__ __forceinline__ void push_track(const DevState<R> *S, int out, const Trk<R> &t, bool has) {
+  if (!__any_sync(0xffffffffu, has)) return;
+  WarpAppend ap;
+  const unsigned rank = ap.add(has, t.type);
+  const unsigned slot = WarpAppend::slot(ap.reserve(S->ctl->cnt[out]), has ? t.type : 0, rank);
+  if (!has) return;
+  if (slot >= S->capacity) {
+    set_status(S->ctl, GV_ERR_STACK_FULL);
+    return;
+  }
+  store_track<R>(S, out, t.type, slot, t.x, t.y, t.z, t.u, t.v, t.w, t.E, t.nlam, t.id, t.ev, t.step,
+                 t.sub | (t.flags << 16));
 }
 
 // The automatic events-in-flight cap (the paper keeps a bounded number of
@@ -537,58 +751,122 @@ __device__ __forceinline__ void primary_cost(const DevState<R> *S, unsigned ev, 
   else atomicAdd(&S->ctl->cost_done, prim_cost(E));
 }
 
-// A track ended: book it against its event; the last one closes the event.
-template <typename R> __device__ __forceinline__ void track_ended(const DevState<R> *S, unsigned ev) {
-  if (atomicSub(&S->evlive[ev], 1u) == 1u) event_closed(S, ev);
+// Live tracks of an event, counted while primaries still wait on the
+// in-flight cap (Ctl::book; once the last primary is out nobody asks).  A
+// final state books its secondaries and its parent's end as one change, so a
+// photoelectric absorption needs no atomic and the event never looks empty
+// in between.  Returns the count before a change by -1, which is 1 where
+// that closed the event (event_closed); 0 for other changes.
+template <typename R> __device__ __forceinline__ unsigned book_live(const DevState<R> *S, unsigned ev, int change) {
+  if (change < 0) return atomicSub(&S->evlive[ev], 1u);
+  if (change > 0) atomicAdd(&S->evlive[ev], static_cast<unsigned>(change));
+  return 0u;
 }
 
-// An interaction request staged in shared memory by the in-block basketizer.
-template <typename R> struct IReq {
-  double x, y, z;
-  unsigned long long id;
-  R E, d0, d1, d2;
-  R u[6];      // u2..u7 of the step
-  unsigned ev, kk;
-  int sub;
-  int tp;      // in: type*3 + process; out: final_state's return code
+// Interaction requests staged in shared memory by the in-block basketizer,
+// one slot per thread, in parts like the queues (each access is then free of
+// bank conflicts): {x, y} {z, id} {E, direction} {event, step, sub, key}
+// {u2, u3} and the final state's return code.
+template <typename R> struct ReqStore {
+  unsigned char *m;
+  int n;  // slots
+  static constexpr int kBytes = 48 + 6 * static_cast<int>(sizeof(R)) + 4;  // per slot
+  __device__ __forceinline__ double2 &xy(int i) const { return reinterpret_cast<double2 *>(m)[i]; }
+  __device__ __forceinline__ double2 &zi(int i) const { return reinterpret_cast<double2 *>(m + 16 * n)[i]; }
+  __device__ __forceinline__ uint4 &info(int i) const { return reinterpret_cast<uint4 *>(m + 32 * n)[i]; }
+  __device__ __forceinline__ V4<R> &dir(int i) const { return reinterpret_cast<V4<R> *>(m + 48 * n)[i]; }
+  __device__ __forceinline__ R &u2(int i) const { return reinterpret_cast<R *>(m + (48 + 4 * sizeof(R)) * n)[i]; }
+  __device__ __forceinline__ R &u3(int i) const { return reinterpret_cast<R *>(m + (48 + 5 * sizeof(R)) * n)[i]; }
+  __device__ __forceinline__ int &ret(int i) const { return reinterpret_cast<int *>(m + (48 + 6 * sizeof(R)) * n)[i]; }
 };
-constexpr int kNKey = 9;
+constexpr int kNKey = kNReqKey;
 
-template <typename R>
-__device__ __forceinline__ void push_survivor(const DevState<R> *S, int out, const Trk<R> &t, bool alive) {
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const bool mine = alive && t.type == q;
-    if (!__ballot_sync(0xffffffffu, mine)) continue;
-    unsigned total;
-    const unsigned slot = warp_reserve(&S->ctl->cnt[out][q], mine ? 1u : 0u, total);
-    if (!mine) continue;
-    if (slot >= S->capacity) {
-      set_status(S->ctl, GV_ERR_STACK_FULL);
-      continue;
-    }
-    store(S->q[out][q], slot, t.x, t.y, t.z, t.u, t.v, t.w, t.E, t.nlam, t.id, t.ev, t.step,
-          t.sub | (t.flags << 16));
+// A primary handed to lane `idx` of the generation: its track, or false if
+// it never entered the box.  Counts per event type by type are left to the
+// caller's warp.
+template <typename R, bool EXT>
+__device__ __forceinline__ bool load_primary(const View<R> &V, const DevState<R> *S, unsigned i, bool book, Trk<R> &t,
+                                             int &note) {
+  Ctl *ctl = S->ctl;
+  const unsigned pi = S->order ? S->order[i] : i;
+  gv_primary p = S->prim[pi];
+  const double e_in = p.E_MeV;  // the budget of the automatic cap is the caller's energy
+  p.event -= S->ev_base;        // the tallies' row (events below the range wrap to a large value)
+  if (p.type < 0 || p.type > 2 || p.event >= S->n_events) {  // caller's device array: check here
+    set_status(ctl, GV_ERR_BAD_ARG);
+    p.type = 0;
+    p.event = 0;
+    p.z = -1.0;
+    p.E_MeV = 0.0;
   }
+  t.type = p.type;
+  t.E = static_cast<R>(p.E_MeV);
+  t.x = p.x; t.y = p.y; t.z = p.z;
+  t.u = static_cast<R>(p.u); t.v = static_cast<R>(p.v); t.w = static_cast<R>(p.w);
+  t.nlam = R(-1);
+  t.id = p.id;
+  t.ev = p.event;
+  t.step = 0;
+  t.flags = kFlagPrimary;
+  t.sub = locate(V.zb, V.geo.nsub, p.z, p.w);
+  const bool in = t.sub >= 0;
+  if (EXT && S->evcnt) {
+    unsigned long long *row = &S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT];
+    atomicAdd(&row[GV_C_TRK_G + t.type], 1ull);
+    if (!in && t.type == 2) atomicAdd(&row[GV_C_EP_ESC], 1ull);
+  }
+  if (!in) {
+    atomicAdd(&S->escape[t.ev], p.E_MeV);
+    if (t.type == 2) note |= kNoteEpEsc;
+  }
+  if (book) {
+    primary_cost(S, t.ev, e_in, in);
+    if (in && atomicAdd(&S->evlive[t.ev], 1u) == 0u) atomicAdd(&ctl->ev_started, 1u);
+  }
+  return in;
 }
 
-// A block-stack secondary written to the output queue (e == nullptr:
-// nothing).  All 32 lanes of a converged warp.
-template <typename R> __device__ __forceinline__ void push_lkid(const DevState<R> *S, int out, const LKid<R> *e) {
-  const int type = e ? e->type : -1;
+// Tracks (and escaped positrons) that a warp's primaries add to the counters.
+__device__ __forceinline__ void count_primaries(unsigned long long *row, bool has, int type, int note) {
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const bool mine = type == q;
-    if (!__ballot_sync(0xffffffffu, mine)) continue;
-    unsigned total;
-    const unsigned slot = warp_reserve(&S->ctl->cnt[out][q], mine ? 1u : 0u, total);
-    if (!mine) continue;
-    if (slot >= S->capacity) {
-      set_status(S->ctl, GV_ERR_STACK_FULL);
-      continue;
-    }
-    store(S->q[out][q], slot, e->x, e->y, e->z, e->u, e->v, e->w, e->E, R(-1), e->id, e->ev, 0u, e->sub);
+  for (int q = 0; q < 3; ++q) wcnt_add(row, GV_C_TRK_G + q, __popc(__ballot_sync(0xffffffffu, has && type == q)));
+  wcnt_add(row, GV_C_EP_ESC, __popc(__ballot_sync(0xffffffffu, has && (note & kNoteEpEsc))));
+}
+
+// Stage the tables, planes, thicknesses, 1/E_i and sub-slab materials into
+// shared memory, with a view of them.  Two block barriers inside.
+template <typename R> __device__ __forceinline__ void stage_tables(const DevState<R> *S, unsigned char *smem, View<R> &sV) {
+  const unsigned tid = threadIdx.x, nt = blockDim.x;
+  const uint4 *src = reinterpret_cast<const uint4 *>(S->view.xs);
+  uint4 *dst = reinterpret_cast<uint4 *>(smem);
+  for (unsigned i = tid; i < S->xs_bytes / 16; i += nt) dst[i] = src[i];
+  const double *zsrc = S->view.zb;
+  double *zdst = reinterpret_cast<double *>(smem + S->xs_bytes);
+  R *tdst = reinterpret_cast<R *>(smem + S->thick_off);
+  const unsigned ns = static_cast<unsigned>(S->view.geo.nsub);
+  for (unsigned i = tid; i <= ns; i += nt) zdst[i] = zsrc[i];
+  for (unsigned i = tid; i < ns; i += nt) tdst[i] = static_cast<R>(zsrc[i + 1] - zsrc[i]);
+  float *idst = reinterpret_cast<float *>(smem + S->xs_bytes + S->zb_bytes);
+  for (unsigned i = tid; i < kGridN; i += nt) idst[i] = S->view.inv_node[i];
+  unsigned char *mdst = smem + S->xs_bytes + S->zb_bytes + kInvNodeBytes;
+  for (unsigned i = tid; i < ns; i += nt) mdst[i] = S->view.smat[i];
+  const uint4 *ssrc = reinterpret_cast<const uint4 *>(S->view.smax);
+  uint4 *sdst = reinterpret_cast<uint4 *>(smem + S->smax_off);
+  for (unsigned i = tid; i < S->smax_bytes / 16; i += nt) sdst[i] = ssrc[i];
+  // the view word by word (one thread copying it was a chain of ~200 loads)
+  static_assert(sizeof(View<R>) % 4 == 0, "copied in words");
+  for (unsigned i = tid; i < sizeof(View<R>) / 4; i += nt)
+    reinterpret_cast<unsigned *>(&sV)[i] = reinterpret_cast<const unsigned *>(&S->view)[i];
+  __syncthreads();
+  if (tid == 0) {
+    sV.xs = reinterpret_cast<const V4<R> *>(smem);
+    sV.zb = zdst;
+    sV.inv_node = idst;
+    sV.smat = mdst;
+    sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
+    sV.thick = tdst;
   }
+  __syncthreads();
 }
 
 // ------------------------------------------------------------------ planning
@@ -601,7 +879,7 @@ __device__ __forceinline__ int claim_queue(int seg) { return seg < 3 ? 2 - seg :
 
 template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   Ctl *c = S->ctl;
-  const unsigned n0 = c->cnt[pn][0], n1 = c->cnt[pn][1], n2 = c->cnt[pn][2];
+  const unsigned n0 = c->cnt[pn][0].n, n1 = c->cnt[pn][1].n, n2 = c->cnt[pn][2].n;
   const unsigned long long live = static_cast<unsigned long long>(n0) + n1 + n2;
   const unsigned rem = S->n_prim - c->prim_next;
   unsigned inj = 0;
@@ -647,6 +925,9 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   c->prim_begin = c->prim_next;
   c->prim_count = inj;
   c->prim_next += inj;
+  // the events' live tracks are asked for only by the in-flight cap, and that
+  // only while primaries wait
+  c->book = S->mode == GV_BATCHED && c->prim_next < S->n_prim && (c->max_in_flight || S->pcost);
   unsigned B = static_cast<unsigned>(S->chunk);
   // With fewer live tracks than the grid has lanes (the first generations of
   // a shower and its tail), a block claims fewer tracks (a multiple of 32)
@@ -668,8 +949,8 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   // once, where the block stack keeps a claim's secondaries stepping in the
   // block (one-round claims there measured slower on small batches)
   c->K = (c->prim_next == S->n_prim && live + inj < S->tail_threshold) ? S->K_tail : S->K_bulk;
-  c->cnt[pn ^ 1][0] = c->cnt[pn ^ 1][1] = c->cnt[pn ^ 1][2] = 0;
-  c->claim = 0;
+  for (int q = 0; q < 3; ++q) c->cnt[pn ^ 1][q].n = 0;
+  c->claim.n = 0;
   for (int r = 0; r < kNClaim; ++r) c->claims[r].n = 0;
   c->blocks_done = 0;
   c->req_n = 0;
@@ -687,7 +968,7 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
 template <typename R> __global__ void init_kernel(const DevState<R> *S) {
   Ctl *c = S->ctl;
   for (int i = 0; i < 2; ++i)
-    for (int q = 0; q < 3; ++q) c->cnt[i][q] = 0;
+    for (int q = 0; q < 3; ++q) c->cnt[i][q].n = 0;
   c->prim_next = 0;
   c->status = 0;
   c->done = 0;
@@ -802,58 +1083,46 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 #define GV_STEP_BOUNDS __launch_bounds__(GV_MAX_BLOCK, sizeof(R) == 4 ? GV_MIN_BLOCKS : 1)
 #endif
 
+//
+// What bounds it: the instruction issue and the latency chains of a round at
+// the two blocks per SM that its registers allow (ncu: issue active 30 %, no
+// memory or FP64 pipe above 25 %).  So the work is cut where few lanes did it:
+// random numbers once per round instead of once per step (run_round), one
+// place that makes secondaries (a stopped positron is a request like any
+// other), counters booked by ballots into words of the warp (a 64-bit
+// shared-memory atomic is a loop), 16-byte track parts, one reservation
+// atomic for the three queues.  2000 x 10 GeV e- in Pb/polystyrene: 7.63 ->
+// 5.39 ms a transport; 1000 x 1 GeV: 1.41 -> 1.13 ms; 300 x 10 GeV in FP64:
+// 13.4 -> 10.8 ms (its arithmetic sits on the FP64 pipe); 2000 x 100 GeV in
+// W/Si with cells: 95.6 -> 65.5 ms.
 template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT>
 __global__ void GV_STEP_BOUNDS
     step_kernel(int parity) {
   const DevState<R> *__restrict__ S = tstate<R>();
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(32) unsigned char smem[];
   __shared__ View<R> sV;
-  __shared__ BlockCnt bc;
+  __shared__ WarpCnt s_wc[GV_MAX_BLOCK / 32];
   __shared__ unsigned s_chunk, s_end[4], s_pb;
   __shared__ unsigned s_slice[kNClaim + 1];
-  __shared__ int s_K, s_last;
+  __shared__ int s_K, s_last, s_book;
   __shared__ unsigned s_B;
   __shared__ int s_ltop;  // the block's secondary stack (local_stack)
-  __shared__ unsigned s_wcnt[SORT ? kNKey : 1][SORT ? 16 : 1];
-  __shared__ unsigned s_walive[SORT ? 16 : 1];
+  __shared__ unsigned s_key[2][kNKey];  // requests per key of this round and the next
   Ctl *ctl = S->ctl;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   // Programmatic dependent launch (pdl): the next generation's blocks may
   // start as soon as this one's finish, stage their tables, and wait for
   // this grid (and its plan) to complete before reading the plan.
   asm volatile("griddepcontrol.launch_dependents;");
   if (ctl->done) return;  // a done flag seen before the wait is final: nothing planned
-  // stage the cross-section tables and the geometry into shared memory
-  {
-    const uint4 *src = reinterpret_cast<const uint4 *>(S->view.xs);
-    uint4 *dst = reinterpret_cast<uint4 *>(smem);
-    for (unsigned i = tid; i < S->xs_bytes / 16; i += blockDim.x) dst[i] = src[i];
-    const double *zsrc = S->view.zb;
-    double *zdst = reinterpret_cast<double *>(smem + S->xs_bytes);
-    const int nz = S->view.geo.nsub + 1;
-    for (int i = tid; i < nz; i += blockDim.x) zdst[i] = zsrc[i];
-    float *idst = reinterpret_cast<float *>(smem + S->xs_bytes + S->zb_bytes);
-    for (int i = tid; i < kGridN; i += blockDim.x) idst[i] = S->view.inv_node[i];
-    unsigned char *mdst = smem + S->xs_bytes + S->zb_bytes + kInvNodeBytes;
-    for (int i = tid; i < S->view.geo.nsub; i += blockDim.x) mdst[i] = S->view.smat[i];
-    {
-      const uint4 *ssrc = reinterpret_cast<const uint4 *>(S->view.smax);
-      uint4 *sdst = reinterpret_cast<uint4 *>(smem + S->smax_off);
-      for (unsigned i = tid; i < S->smax_bytes / 16; i += blockDim.x) sdst[i] = ssrc[i];
-    }
-    if (tid == 0) {
-      sV = S->view;
-      sV.xs = reinterpret_cast<const V4<R> *>(smem);
-      sV.zb = zdst;
-      sV.inv_node = idst;
-      sV.smat = mdst;
-      sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
-    }
-    if (tid < 16) bc.c[tid] = 0;
-  }
+  unsigned long long *const row = s_wc[tid >> 5];
+  if (lane < 16) row[lane] = 0ull;
+  if (tid < 2 * kNKey) s_key[tid / kNKey][tid % kNKey] = 0u;
+  stage_tables(S, smem, sV);
   // the previous generation, and its plan, complete before the plan is read
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (ctl->done) return;  // uniform: nothing planned for this generation
+  const bool block_claims = SORT || S->claim_chunks == 0;
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) s_end[i] = ctl->chunk_end[i];
     for (int r = 0; r <= kNClaim; ++r)
@@ -861,23 +1130,29 @@ __global__ void GV_STEP_BOUNDS
     s_pb = ctl->prim_begin;
     s_K = ctl->K;
     s_B = ctl->chunk_B;
+    s_book = ctl->book;
     s_ltop = 0;
+    // the first claim; each later one is issued before the previous claim's survivors go out
+    if (block_claims) s_chunk = atomicAdd(&ctl->claim.n, 1u);
   }
   __syncthreads();
   const View<R> &V = sV;
   const int in = parity, out = parity ^ 1;
   const unsigned cap = static_cast<unsigned>(S->capacity);
-  const unsigned n_in[3] = {min(ctl->cnt[in][0], cap), min(ctl->cnt[in][1], cap), min(ctl->cnt[in][2], cap)};
   const unsigned n_prim_gen = ctl->prim_count;
   // With several rounds per claim, the secondaries made in a round stay in
   // the block and fill its idle lanes in the next rounds (local_stack).
   const bool use_local = SORT && S->local_stack && s_K > 1;
+  const bool book = s_book != 0;
   LocalStack<R> lstk;
-  lstk.e = reinterpret_cast<LKid<R> *>(smem + S->smem_lk_off);
+  lstk.e = smem + S->smem_lk_off;
   lstk.top = &s_ltop;
   lstk.cap = static_cast<int>(blockDim.x);
-  int w_slice = 0;
-  {
+  ReqStore<R> req;
+  req.m = smem + S->smem_req_off;
+  req.n = static_cast<int>(blockDim.x);
+  int w_slice = 0, buf = 0;
+  if (!block_claims) {
     unsigned smid;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
     w_slice = static_cast<int>((smid * 4u + ((tid >> 5) & 3u)) % kNClaim);
@@ -887,11 +1162,6 @@ __global__ void GV_STEP_BOUNDS
   pend.sum = R(0);
   pend.comp = R(0);
   Pending<R> *const pd = MERGE ? &pend : nullptr;
-  const bool block_claims = SORT || S->claim_chunks == 0;
-  if (block_claims) {  // the first claim; each later one is issued before the previous claim's survivors go out
-    if (tid == 0) s_chunk = atomicAdd(&ctl->claim, 1u);
-    __syncthreads();
-  }
   for (;;) {
     // Work claiming: with the basketizer a chunk is one block (its step loop
     // syncs the block); without it every warp claims its own 32-track chunks
@@ -899,14 +1169,15 @@ __global__ void GV_STEP_BOUNDS
     unsigned chunk, idx;
     if (block_claims) {
       chunk = s_chunk;
-      __syncthreads();
+      // (the basketizer's own barriers stand between this read and the next write)
+      if (!SORT) __syncthreads();
     } else {
       // The chunk range is split into kNClaim slices, each with its own
       // counter in its own cache line: a warp draws from its SM's slice and
       // moves on when that slice is spent, so no single address takes every
       // claim of the generation.
       unsigned c0 = 0;
-      if ((tid & 31) == 0) {
+      if (lane == 0) {
         c0 = 0xffffffffu;
         for (int k = 0; k < kNClaim; ++k) {
           const int r = (w_slice + k) % kNClaim;
@@ -927,249 +1198,192 @@ __global__ void GV_STEP_BOUNDS
     int qsel = 0;
     while (chunk >= s_end[qsel]) ++qsel;
     {
-      const bool per_block = SORT || S->claim_chunks == 0;
-      const unsigned csize = per_block ? s_B : 32u;
-      idx = (chunk - (qsel ? s_end[qsel - 1] : 0u)) * csize + (per_block ? tid : (tid & 31));
-      if (per_block && static_cast<unsigned>(tid) >= csize) idx = 0xffffffffu;
+      const unsigned csize = block_claims ? s_B : 32u;
+      idx = (chunk - (qsel ? s_end[qsel - 1] : 0u)) * csize + (block_claims ? tid : lane);
+      if (block_claims && static_cast<unsigned>(tid) >= csize) idx = 0xffffffffu;
     }
     qsel = claim_queue(qsel);
     Trk<R> t;
+    t.type = 0;
+    t.ev = 0;
     bool alive = false;
     if (qsel < 3) {
-      if (idx < n_in[qsel]) {
-        const Queue<R> &q = S->q[in][qsel];
-        t.x = q.x[idx]; t.y = q.y[idx]; t.z = q.z[idx];
-        t.u = q.u[idx]; t.v = q.v[idx]; t.w = q.w[idx];
-        t.E = q.E[idx]; t.nlam = q.nlam[idx];
-        t.id = q.id[idx]; t.ev = q.ev[idx]; t.step = q.step[idx];
-        const int sf = q.sf[idx];
-        t.sub = sf & 0xffff;
-        t.flags = sf >> 16;
-        t.type = qsel;
+      if (idx < min(ctl->cnt[in][qsel].n, cap)) {
+        load_track<R>(S, in, qsel, idx, t);
         alive = true;
         GV_CHECK(&ctl->status, t.sub >= 0 && t.sub < V.geo.nsub && t.ev < S->n_events && t.E >= R(0));
       }
-    } else if (idx < n_prim_gen) {
-      const unsigned i = s_pb + idx;
-      const unsigned pi = S->order ? S->order[i] : i;
-      gv_primary p = S->prim[pi];
-      const double e_in = p.E_MeV;  // the budget of the automatic cap is the caller's energy
-      p.event -= S->ev_base;  // the tallies' row (events below the range wrap to a large value)
-      if (p.type < 0 || p.type > 2 || p.event >= S->n_events) {  // caller's device array: check here
-        set_status(ctl, GV_ERR_BAD_ARG);
-        p.type = 0;
-        p.event = 0;
-        p.z = -1.0;
-        p.E_MeV = 0.0;
-      }
-      t.type = p.type;
-      t.E = static_cast<R>(p.E_MeV);
-      t.x = p.x; t.y = p.y; t.z = p.z;
-      t.u = static_cast<R>(p.u); t.v = static_cast<R>(p.v); t.w = static_cast<R>(p.w);
-      t.nlam = R(-1);
-      t.id = p.id;
-      t.ev = p.event;
-      t.step = 0;
-      t.flags = kFlagPrimary;
-      t.sub = locate(V.zb, V.geo.nsub, p.z, p.w);
-      count<R, EXT>(S, &bc, t.ev, GV_C_TRK_G + t.type);
-      if (t.sub < 0) {
-        atomicAdd(&S->escape[t.ev], p.E_MeV);
-        if (t.type == 2) count<R, EXT>(S, &bc, t.ev, GV_C_EP_ESC);
-        primary_cost(S, t.ev, e_in, false);
-      } else {
-        alive = true;
-        primary_cost(S, t.ev, e_in, true);
-        if (atomicAdd(&S->evlive[t.ev], 1u) == 0u) atomicAdd(&ctl->ev_started, 1u);
-      }
+    } else {
+      const bool has = idx < n_prim_gen;
+      int note = 0;
+      if (has) alive = load_primary<R, EXT>(V, S, s_pb + idx, book, t, note);
+      count_primaries(row, has, t.type, note);
     }
     const int K = s_K;
-    unsigned ended_prev = 0u;  // evlive before this lane's last track ended (1: it closed its event)
+    unsigned ended_own = 0u, ended_req = 0u;  // evlive before this lane's last bookings of an end (1: the event closed)
+    unsigned ev_req = 0u;
     for (int kk = 0; kk < K; ++kk) {
       // (with the basketizer the block leaves the loop together, after the
       // count barrier below shows that no lane was alive)
       if (!SORT && !__any_sync(0xffffffffu, alive)) break;
-      if (use_local && kk > 0 && !alive) {  // take up a secondary of an earlier round
-        const int i = atomicSub(&s_ltop, 1) - 1;
-        if (i >= 0 && i < lstk.cap) {
-          const LKid<R> &e = lstk.e[i];
-          t.x = e.x; t.y = e.y; t.z = e.z;
-          t.u = e.u; t.v = e.v; t.w = e.w;
-          t.E = e.E;
-          t.nlam = R(-1);
-          t.id = e.id;
-          t.ev = e.ev;
-          t.step = 0;
-          t.sub = e.sub;
-          t.flags = 0;
-          t.type = e.type;
-          alive = true;
+      if (use_local && kk > 0) {  // idle lanes take up secondaries of earlier rounds
+        const unsigned idle = __ballot_sync(0xffffffffu, !alive);
+        if (idle) {
+          int top = 0;
+          if (lane == 0) top = atomicSub(&s_ltop, __popc(idle));
+          top = __shfl_sync(0xffffffffu, top, 0);
+          const int i = top - 1 - __popc(idle & ((1u << lane) - 1u));
+          if (!alive && i >= 0 && i < lstk.cap) {
+            lstk.get(i, t);
+            alive = true;
+          }
         }
       }
       const bool was_alive = alive;
-      Kids<R> kids;
-      kids.n = 0;
-      uint32_t kstep = 0;
-      int proc = -1, lim = -1;
-      R u[8];
       // Along-step part.  With the basketizer a lane keeps stepping (boundary-
       // and continuous-limited steps need no final state) until its track is
-      // due a discrete interaction, ends, or has taken along_steps steps; the
-      // block then baskets the interactions.  Step tallies stay per lane and
-      // are summed per warp afterwards.
-      unsigned n_st = 0, n_geom = 0, n_iter = 0;
-      // photons cross layers in runs of boundary-limited steps; charged tracks
-      // are stopped more often by their continuous-loss limit: each type has
-      // its own budget (measured best at 5 and 3 on the benchmark)
-      const int inner = SORT ? (t.type == 0 ? S->along_steps_g : S->along_steps) : 1;
-      for (int m = 0; m < inner && alive && proc < 0; ++m) {
-        ++n_iter;
-        const uint32_t before = t.step;
-        alive = step_track<R, FIELD, OPTS, EXT>(V, S, t, kids, kstep, &bc, proc, u, lim, pd) != 0;
-        // NaN energy, or a non-finite z (tested on its exponent bits: an FP64
-        // comparison would take the FP64 pipe)
-        if (!(t.E == t.E) || (__double2hiint(t.z) & 0x7ff00000) == 0x7ff00000) {
-          set_status(ctl, GV_ERR_NUMERIC);
-          alive = false;
-          proc = -1;
-        }
-        if (t.step != before) {
-          ++n_st;
-          n_geom += lim == 0 ? 1u : 0u;
-        }
-      }
-      if (!SORT && alive && proc >= 0) {  // final state in place (warp-divergent across processes)
-        R d[3] = {t.u, t.v, t.w};
-        const int r = final_state<R, OPTS, EXT>(V, S, &bc, t.type, proc, t.E, d, u, kids, t.ev, t.sub, t.x, t.y, t.id, kstep, pd);
-        if (r >= 0) {
-          t.u = d[0]; t.v = d[1]; t.w = d[2];
-          t.flags |= kFlagInteracted;
-          alive = r != 0;
-        }
-      }
-      push_kids<R, EXT>(S, out, parent_of(t), kids, kstep, &bc);
-      if (MERGE) warp_flush(S, pend);
-      {  // step counters, one shared-memory atomic per warp and kind
-        const unsigned wst = __reduce_add_sync(0xffffffffu, n_st);
-        const unsigned wiq = __reduce_max_sync(0xffffffffu, n_iter);
-        if (wst) {
-          const unsigned wg = __reduce_add_sync(0xffffffffu, t.type == 0 ? n_st : 0u);
-          const unsigned we = __reduce_add_sync(0xffffffffu, t.type == 1 ? n_st : 0u);
-          const unsigned wx = __reduce_add_sync(0xffffffffu, (n_st && proc >= 0) ? 1u : 0u);
-          const unsigned wb = __reduce_add_sync(0xffffffffu, n_geom);
-          if ((tid & 31) == 0) {
-            atomicAdd(&bc.c[GV_C_STEPS], static_cast<unsigned long long>(wst));
-            if (wg) atomicAdd(&bc.c[GV_C_STEPS_G], static_cast<unsigned long long>(wg));
-            if (we) atomicAdd(&bc.c[GV_C_STEPS_EM], static_cast<unsigned long long>(we));
-            if (wst - wg - we) atomicAdd(&bc.c[GV_C_STEPS_EP], static_cast<unsigned long long>(wst - wg - we));
-            if (wx) atomicAdd(&bc.c[GV_C_DISCRETE], static_cast<unsigned long long>(wx));
-            if (wb) atomicAdd(&bc.c[GV_C_GEOM], static_cast<unsigned long long>(wb));
-          }
-        }
-        if ((tid & 31) == 0 && wiq) atomicAdd(&bc.c[GV_C_LANE_SLOTS], 32ull * wiq);  // idle-lane fraction
-      }
-      if (SORT) {
-        // Basketizer: counting sort of this step's interaction requests by
-        // (type, process) -- warp ballots, a prefix sum over keys and warps,
-        // one slot each -- so every warp runs a single final-state model.
-        // Three block barriers per step: counts, requests, results.
-        IReq<R> *req = reinterpret_cast<IReq<R> *>(smem + S->smem_req_off);
-        const int key = (alive && proc >= 0) ? t.type * 3 + proc : -1;
-        const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-        unsigned rank = 0;
-#pragma unroll
-        for (int k = 0; k < kNKey; ++k) {
-          const unsigned m = __ballot_sync(0xffffffffu, key == k);
-          if (lane == 0) s_wcnt[k][warp] = __popc(m);
-          if (key == k) rank = __popc(m & ((1u << lane) - 1u));
-        }
-        const unsigned ma = __ballot_sync(0xffffffffu, was_alive);
-        if (lane == 0) s_walive[warp] = ma;
-        __syncthreads();
-        if (use_local && tid == 0 && s_ltop < 0) s_ltop = 0;  // pops of an empty stack
-        unsigned any = 0;
-        for (int w = 0; w < nw; ++w) any |= s_walive[w];
-        if (!any) break;  // uniform: no lane of the block was alive this step
-        // lane k < kNKey: requests of key k in the block and in warps before this one
-        unsigned ck = 0, part = 0;
-        if (lane < kNKey) {
-          for (int w = 0; w < nw; ++w) {
-            const unsigned c = s_wcnt[lane][w];
-            ck += c;
-            part += (w < warp) ? c : 0u;
-          }
-        }
-        unsigned incl = ck;
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-          const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const unsigned start = incl - ck + part;  // first slot of key `lane` for this warp
-        const unsigned nreq = __shfl_sync(0xffffffffu, incl, kNKey - 1);
-        const unsigned mine = __shfl_sync(0xffffffffu, start, key >= 0 ? key : 0);
-        const unsigned slot = key >= 0 ? mine + rank : 0u;
+      // due a discrete interaction, ends, or has taken its type's budget of
+      // steps (photons cross layers in runs of boundary-limited steps; charged
+      // tracks are stopped more often by their continuous-loss limit: measured
+      // best at 5 and 3 on the benchmark); the block then baskets the
+      // interactions.
+      uint32_t kstep;
+      R u2 = R(0), u3 = R(0);
+      Run<R> run;
+      const int key = run_round<R, FIELD, OPTS, EXT>(V, S, t, alive, SORT ? S->along_steps_g : 1,
+                                                     SORT ? S->along_steps : 1, kstep, u2, u3, run, pd);
+      count_round(row, run, t.type, key >= 0 && key != kKeyRest);
+      bool own_end = was_alive && !alive && key < 0;  // ended without a final state
+      if (!SORT) {  // final state in place (warp-divergent across processes)
+        Kids<R> kids;
+        kids.n = 0;
+        int np = 0, na = 0, change = own_end ? -1 : 0;
         if (key >= 0) {
-          IReq<R> &q = req[slot];
-          q.x = t.x; q.y = t.y; q.z = t.z;
-          q.id = t.id;
-          q.E = t.E; q.d0 = t.u; q.d1 = t.v; q.d2 = t.w;
-#pragma unroll
-          for (int j = 0; j < 6; ++j) q.u[j] = u[2 + j];
-          q.ev = t.ev;
-          q.kk = kstep;
-          q.sub = t.sub;
-          q.tp = key;
+          R d[3] = {t.u, t.v, t.w};
+          const int r = final_state<R, OPTS, EXT>(V, S, key, t.E, d, u2, u3, kids, t.ev, t.sub, t.x, t.y, t.id, kstep, np,
+                                                  na, pd);
+          if (r >= 0) {
+            t.u = d[0]; t.v = d[1]; t.w = d[2];
+            t.flags |= kFlagInteracted;
+            alive = r != 0;
+          }
+          change = kids.n - (r == 0 ? 1 : 0);
         }
-        __syncthreads();
+        wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
+        wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
+        if (book && book_live(S, t.ev, change) == 1u) event_closed(S, t.ev);
+        push_kids<R, EXT>(S, out, Parent{t.x, t.y, t.z, t.id, t.ev, t.sub}, kids, kstep, row);
+        if (MERGE) warp_flush(S, pend);
+        continue;
+      }
+      if (MERGE) warp_flush(S, pend);
+      // Basketizer: counting sort of this step's interaction requests by
+      // (type, process), so every warp runs a single final-state model.
+      // Three block barriers per round: counts, requests, results.  A warp
+      // ranks its requests key by key (the keys it has: one to three), and
+      // one lane per key adds its count to the block's.
+      unsigned rank = 0, base = 0;
+      int leader = 0;
+      for (unsigned rest = __ballot_sync(0xffffffffu, key >= 0); rest;) {
+        const int l = __ffs(rest) - 1;
+        const unsigned m = __ballot_sync(0xffffffffu, key == __shfl_sync(0xffffffffu, key, l));
+        if (m >> lane & 1u) {
+          rank = __popc(m & ((1u << lane) - 1u));
+          leader = l;
+          if (lane == l) base = __popc(m);
+        }
+        rest &= ~m;
+      }
+      if (base) base = atomicAdd(&s_key[buf][key], base);
+      base = __shfl_sync(0xffffffffu, base, leader);
+      if (!__syncthreads_or(was_alive)) break;  // uniform: no lane of the block was alive this step
+      if (use_local && tid == 0 && s_ltop < 0) s_ltop = 0;  // pops of an empty stack
+      if (tid < kNKey) s_key[buf ^ 1][tid] = 0u;
+      const unsigned ck = lane < kNKey ? s_key[buf][lane] : 0u;
+      unsigned incl = ck;
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const unsigned nreq = __shfl_sync(0xffffffffu, incl, kNKey - 1);
+      const unsigned first = __shfl_sync(0xffffffffu, incl - ck, key >= 0 ? key : 0);
+      const int slot = static_cast<int>(first + base + rank);
+      buf ^= 1;
+      if (key >= 0) {
+        req.xy(slot) = make_double2(t.x, t.y);
+        req.zi(slot) = make_double2(t.z, i2d(t.id));
+        req.info(slot) = make_uint4(t.ev, kstep, static_cast<unsigned>(t.sub), static_cast<unsigned>(key));
+        req.dir(slot) = V4<R>{t.u, t.v, t.w, t.E};
+        req.u2(slot) = u2;
+        req.u3(slot) = u3;
+      }
+      __syncthreads();
+      {
         Kids<R> kb;
         kb.n = 0;
         Parent par;
         uint32_t pk = 0;
+        int np = 0, na = 0;
         if (static_cast<unsigned>(tid) < nreq) {
-          IReq<R> &q = req[tid];
-          R uu[8] = {R(0), R(0), q.u[0], q.u[1], q.u[2], q.u[3], q.u[4], q.u[5]};
-          R d[3] = {q.d0, q.d1, q.d2};
-          R e = q.E;
-          const int ty = q.tp / 3;
-          const int r = final_state<R, OPTS, EXT>(V, S, &bc, ty, q.tp - 3 * ty, e, d, uu, kb, q.ev, q.sub, q.x, q.y, q.id, q.kk);
-          par.x = q.x; par.y = q.y; par.z = q.z;
-          par.id = q.id;
-          par.ev = q.ev;
-          par.sub = q.sub;
-          pk = q.kk;
-          q.E = e; q.d0 = d[0]; q.d1 = d[1]; q.d2 = d[2];
-          q.tp = r;
-        }
-        push_kids<R, EXT>(S, out, par, kb, pk, &bc, use_local ? &lstk : nullptr);
-        __syncthreads();
-        if (key >= 0) {
-          const IReq<R> &q = req[slot];
-          if (q.tp >= 0) {
-            t.E = q.E; t.u = q.d0; t.v = q.d1; t.w = q.d2;
-            t.flags |= kFlagInteracted;
-            alive = q.tp != 0;
+          const double2 a = req.xy(tid), c = req.zi(tid);
+          const uint4 g = req.info(tid);
+          const V4<R> dE = req.dir(tid);
+          par.x = a.x; par.y = a.y; par.z = c.x;
+          par.id = d2i(c.y);
+          par.ev = g.x;
+          par.sub = static_cast<int>(g.z);
+          pk = g.y;
+          R d[3] = {dE.x, dE.y, dE.z};
+          R e = dE.w;
+          const int r = final_state<R, OPTS, EXT>(V, S, static_cast<int>(g.w), e, d, req.u2(tid), req.u3(tid), kb, par.ev,
+                                                  par.sub, par.x, par.y, par.id, pk, np, na);
+          req.dir(tid) = V4<R>{d[0], d[1], d[2], e};
+          req.ret(tid) = r;
+          if (book) {
+            ended_req = book_live(S, par.ev, kb.n - (r == 0 ? 1 : 0));
+            ev_req = par.ev;
           }
         }
+        wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
+        wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
+        push_kids<R, EXT>(S, out, par, kb, pk, row, use_local ? &lstk : nullptr);
       }
-      if (was_alive && !alive) {
-        if (kk + 1 < K) track_ended(S, t.ev);
-        else ended_prev = atomicSub(&S->evlive[t.ev], 1u);  // read after the survivors are out
+      __syncthreads();
+      if (key >= 0 && key != kKeyRest) {
+        const int r = req.ret(slot);
+        if (r >= 0) {
+          const V4<R> dE = req.dir(slot);
+          t.E = dE.w; t.u = dE.x; t.v = dE.y; t.w = dE.z;
+          t.flags |= kFlagInteracted;
+          alive = r != 0;
+        }
+      }
+      if (book) {  // the last round's are read after the survivors are out
+        if (own_end) ended_own = book_live(S, t.ev, -1);
+        if (kk + 1 < K) {
+          if (ended_own == 1u) event_closed(S, t.ev);
+          if (ended_req == 1u) event_closed(S, ev_req);
+          ended_own = ended_req = 0u;
+        }
       }
     }
     // the next claim's atomic and the event count's are in flight while the
     // survivors are written
     unsigned next_chunk = 0u;
-    if (block_claims && tid == 0) next_chunk = atomicAdd(&ctl->claim, 1u);
+    if (block_claims && tid == 0) next_chunk = atomicAdd(&ctl->claim.n, 1u);
     if (MERGE) warp_flush(S, pend);  // nothing stays pending past a claim
-    push_survivor(S, out, t, alive);
-    if (ended_prev == 1u) event_closed(S, t.ev);
+    push_track(S, out, t, alive);
+    if (ended_own == 1u) event_closed(S, t.ev);
+    if (ended_req == 1u) event_closed(S, ev_req);
     if (use_local) {  // what is left on the block's stack goes to the next generation
       __syncthreads();
       const int n = max(0, min(s_ltop, lstk.cap));
-      for (int base = 0; base < n; base += blockDim.x) {
-        const int i = base + tid;
-        push_lkid(S, out, i < n ? &lstk.e[i] : static_cast<const LKid<R> *>(nullptr));
+      for (int b = 0; b < n; b += blockDim.x) {
+        Trk<R> k;
+        k.type = 0;
+        if (b + tid < n) lstk.get(b + tid, k);
+        push_track(S, out, k, b + tid < n);
       }
       __syncthreads();
       if (tid == 0) s_ltop = 0;
@@ -1179,9 +1393,13 @@ __global__ void GV_STEP_BOUNDS
       __syncthreads();
     }
   }
-  // flush block counters; the last block plans the next generation
+  // flush the warps' counters; the last block plans the next generation
   __syncthreads();
-  if (tid < 16 && bc.c[tid]) atomicAdd(&ctl->counters[tid], bc.c[tid]);
+  if (tid < 16) {
+    unsigned long long v = 0ull;
+    for (unsigned w = 0; w < blockDim.x / 32; ++w) v += s_wc[w][tid];
+    if (v) atomicAdd(&ctl->counters[tid], v);
+  }
   __syncthreads();
   if (tid == 0) {
     __threadfence();
@@ -1209,22 +1427,25 @@ __global__ void GV_STEP_BOUNDS
 // Hand the tracks due an interaction to the interaction kernel.  All 32
 // lanes of a converged warp.
 template <typename R>
-__device__ void emit_requests(const DevState<R> *S, const Trk<R> &t, bool hand, int proc, uint32_t kstep,
-                              const R *u) {
-  if (!__ballot_sync(0xffffffffu, hand)) return;
+__device__ void emit_requests(const DevState<R> *S, const Trk<R> &t, int key, uint32_t kstep, R u2, R u3) {
+  const bool hand = key >= 0;
+  const unsigned mh = __ballot_sync(0xffffffffu, hand);
+  if (!mh) return;
   Ctl *ctl = S->ctl;
-  unsigned total;
-  const unsigned slot = warp_reserve(&ctl->req_n, hand ? 1u : 0u, total);
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  unsigned base = 0;
+  if (lane == 0) base = atomicAdd(&ctl->req_n, __popc(mh));
+  const unsigned slot = __shfl_sync(0xffffffffu, base, 0) + __popc(mh & lt);
   const bool ok = hand && slot < S->req_cap;
   if (hand && !ok) set_status(ctl, GV_ERR_STACK_FULL);
-  const int key = t.type * 3 + proc;
   if (ok) {
     GReq<R> &q = S->req[slot];
     q.x = t.x; q.y = t.y; q.z = t.z;
     q.id = t.id;
     q.E = t.E; q.d0 = t.u; q.d1 = t.v; q.d2 = t.w;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) q.u[j] = u[2 + j];
+    q.u2 = u2;
+    q.u3 = u3;
     q.ev = t.ev;
     q.kk = kstep;
     q.sf = t.sub | (t.flags << 16);
@@ -1232,11 +1453,12 @@ __device__ void emit_requests(const DevState<R> *S, const Trk<R> &t, bool hand, 
   }
 #pragma unroll
   for (int k = 0; k < kNReqKey; ++k) {
-    const bool mine = ok && key == k;
-    if (!__ballot_sync(0xffffffffu, mine)) continue;
-    unsigned tk;
-    const unsigned pos = warp_reserve(&ctl->key_n[k], mine ? 1u : 0u, tk);
-    if (mine) S->keyidx[static_cast<size_t>(k) * S->req_cap + pos] = slot;
+    const unsigned m = __ballot_sync(0xffffffffu, ok && key == k);
+    if (!m) continue;
+    unsigned b = 0;
+    if (lane == 0) b = atomicAdd(&ctl->key_n[k], __popc(m));
+    b = __shfl_sync(0xffffffffu, b, 0);
+    if (m >> lane & 1u) S->keyidx[static_cast<size_t>(k) * S->req_cap + b + __popc(m & lt)] = slot;
   }
 }
 
@@ -1245,170 +1467,75 @@ template <typename R>
 #define GV_ALONG_MIN_BLOCKS 2
 #endif
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? GV_ALONG_MIN_BLOCKS : 2) along_kernel(const DevState<R> *__restrict__ S, int parity) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(32) unsigned char smem[];
   __shared__ View<R> sV;
-  __shared__ BlockCnt bc;
-  __shared__ unsigned s_chunk, s_end[4], s_pb;
-  __shared__ int s_K;
+  __shared__ WarpCnt s_wc[8];
+  __shared__ unsigned s_chunk;
   Ctl *ctl = S->ctl;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   if (ctl->done) return;
-  {  // tables, planes, 1/E_i and sub-slab materials into shared memory
-    const uint4 *src = reinterpret_cast<const uint4 *>(S->view.xs);
-    uint4 *dst = reinterpret_cast<uint4 *>(smem);
-    for (unsigned i = tid; i < S->xs_bytes / 16; i += blockDim.x) dst[i] = src[i];
-    const double *zsrc = S->view.zb;
-    double *zdst = reinterpret_cast<double *>(smem + S->xs_bytes);
-    const int nz = S->view.geo.nsub + 1;
-    for (int i = tid; i < nz; i += blockDim.x) zdst[i] = zsrc[i];
-    float *idst = reinterpret_cast<float *>(smem + S->xs_bytes + S->zb_bytes);
-    for (int i = tid; i < kGridN; i += blockDim.x) idst[i] = S->view.inv_node[i];
-    unsigned char *mdst = smem + S->xs_bytes + S->zb_bytes + kInvNodeBytes;
-    for (int i = tid; i < S->view.geo.nsub; i += blockDim.x) mdst[i] = S->view.smat[i];
-    {
-      const uint4 *ssrc = reinterpret_cast<const uint4 *>(S->view.smax);
-      uint4 *sdst = reinterpret_cast<uint4 *>(smem + S->smax_off);
-      for (unsigned i = tid; i < S->smax_bytes / 16; i += blockDim.x) sdst[i] = ssrc[i];
-    }
-    if (tid == 0) {
-      sV = S->view;
-      sV.xs = reinterpret_cast<const V4<R> *>(smem);
-      sV.zb = zdst;
-      sV.inv_node = idst;
-      sV.smat = mdst;
-      sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
-      for (int i = 0; i < 4; ++i) s_end[i] = ctl->chunk_end[i];
-      s_pb = ctl->prim_begin;
-      s_K = ctl->K;
-    }
-    if (tid < 16) bc.c[tid] = 0;
-  }
-  __syncthreads();
+  unsigned long long *const row = s_wc[tid >> 5];
+  if (lane < 16) row[lane] = 0ull;
+  stage_tables(S, smem, sV);
   const View<R> &V = sV;
   const int in = parity, out = parity ^ 1;
   const unsigned cap = static_cast<unsigned>(S->capacity);
-  const unsigned n_in[3] = {min(ctl->cnt[in][0], cap), min(ctl->cnt[in][1], cap), min(ctl->cnt[in][2], cap)};
-  const unsigned n_prim_gen = ctl->prim_count;
+  const unsigned n_prim_gen = ctl->prim_count, n_chunks = ctl->chunk_end[3];
+  const bool book = ctl->book != 0;
   for (;;) {
-    if (tid == 0) s_chunk = atomicAdd(&ctl->claim, 1u);
+    if (tid == 0) s_chunk = atomicAdd(&ctl->claim.n, 1u);
     __syncthreads();
     const unsigned chunk = s_chunk;
     __syncthreads();
-    if (chunk >= s_end[3]) break;
+    if (chunk >= n_chunks) break;
     int qsel = 0;
-    while (chunk >= s_end[qsel]) ++qsel;
-    const unsigned idx = (chunk - (qsel ? s_end[qsel - 1] : 0u)) * blockDim.x + tid;
+    while (chunk >= ctl->chunk_end[qsel]) ++qsel;
+    const unsigned idx = (chunk - (qsel ? ctl->chunk_end[qsel - 1] : 0u)) * blockDim.x + tid;
     qsel = claim_queue(qsel);
     Trk<R> t;
+    t.type = 0;
+    t.ev = 0;
     bool alive = false;
     if (qsel < 3) {
-      if (idx < n_in[qsel]) {
-        const Queue<R> &q = S->q[in][qsel];
-        t.x = q.x[idx]; t.y = q.y[idx]; t.z = q.z[idx];
-        t.u = q.u[idx]; t.v = q.v[idx]; t.w = q.w[idx];
-        t.E = q.E[idx]; t.nlam = q.nlam[idx];
-        t.id = q.id[idx]; t.ev = q.ev[idx]; t.step = q.step[idx];
-        const int sf = q.sf[idx];
-        t.sub = sf & 0xffff;
-        t.flags = sf >> 16;
-        t.type = qsel;
+      if (idx < min(ctl->cnt[in][qsel].n, cap)) {
+        load_track<R>(S, in, qsel, idx, t);
         alive = true;
         GV_CHECK(&ctl->status, t.sub >= 0 && t.sub < V.geo.nsub && t.ev < S->n_events && t.E >= R(0));
       }
-    } else if (idx < n_prim_gen) {
-      const unsigned i = s_pb + idx;
-      const unsigned pi = S->order ? S->order[i] : i;
-      gv_primary p = S->prim[pi];
-      const double e_in = p.E_MeV;  // the budget of the automatic cap is the caller's energy
-      p.event -= S->ev_base;  // the tallies' row (events below the range wrap to a large value)
-      if (p.type < 0 || p.type > 2 || p.event >= S->n_events) {  // caller's device array: check here
-        set_status(ctl, GV_ERR_BAD_ARG);
-        p.type = 0;
-        p.event = 0;
-        p.z = -1.0;
-        p.E_MeV = 0.0;
-      }
-      t.type = p.type;
-      t.E = static_cast<R>(p.E_MeV);
-      t.x = p.x; t.y = p.y; t.z = p.z;
-      t.u = static_cast<R>(p.u); t.v = static_cast<R>(p.v); t.w = static_cast<R>(p.w);
-      t.nlam = R(-1);
-      t.id = p.id;
-      t.ev = p.event;
-      t.step = 0;
-      t.flags = kFlagPrimary;
-      t.sub = locate(V.zb, V.geo.nsub, p.z, p.w);
-      count(S, &bc, t.ev, GV_C_TRK_G + t.type);
-      if (t.sub < 0) {
-        atomicAdd(&S->escape[t.ev], p.E_MeV);
-        if (t.type == 2) count(S, &bc, t.ev, GV_C_EP_ESC);
-        primary_cost(S, t.ev, e_in, false);
-      } else {
-        alive = true;
-        primary_cost(S, t.ev, e_in, true);
-        if (atomicAdd(&S->evlive[t.ev], 1u) == 0u) atomicAdd(&ctl->ev_started, 1u);
-      }
+    } else {
+      const bool has = idx < n_prim_gen;
+      int note = 0;
+      if (has) alive = load_primary<R, true>(V, S, ctl->prim_begin + idx, book, t, note);
+      count_primaries(row, has, t.type, note);
     }
-    const int K = s_K;
+    const int K = ctl->K;
     for (int kk = 0; kk < K; ++kk) {
       if (!__any_sync(0xffffffffu, alive)) break;
       const bool was_alive = alive;
-      Kids<R> kids;
-      kids.n = 0;
-      uint32_t kstep = 0;
-      int proc = -1, lim = -1;
-      R u[8];
-      unsigned n_st = 0, n_geom = 0, n_iter = 0;
-      const int inner = t.type == 0 ? S->along_steps_g : S->along_steps;
-      for (int m = 0; m < inner && alive && proc < 0; ++m) {
-        ++n_iter;
-        const uint32_t before = t.step;
-        alive = step_track<R, true, true, true>(V, S, t, kids, kstep, &bc, proc, u, lim, static_cast<Pending<R> *>(nullptr)) != 0;
-        if (!(t.E == t.E) || (__double2hiint(t.z) & 0x7ff00000) == 0x7ff00000) {
-          set_status(ctl, GV_ERR_NUMERIC);
-          alive = false;
-          proc = -1;
-        }
-        if (t.step != before) {
-          ++n_st;
-          n_geom += lim == 0 ? 1u : 0u;
-        }
-      }
-      push_kids(S, out, parent_of(t), kids, kstep, &bc);
-      {  // step counters, one shared-memory atomic per warp and kind
-        const unsigned wst = __reduce_add_sync(0xffffffffu, n_st);
-        const unsigned wiq = __reduce_max_sync(0xffffffffu, n_iter);
-        if (wst) {
-          const unsigned wg = __reduce_add_sync(0xffffffffu, t.type == 0 ? n_st : 0u);
-          const unsigned we = __reduce_add_sync(0xffffffffu, t.type == 1 ? n_st : 0u);
-          const unsigned wx = __reduce_add_sync(0xffffffffu, (n_st && alive && proc >= 0) ? 1u : 0u);
-          const unsigned wb = __reduce_add_sync(0xffffffffu, n_geom);
-          if ((tid & 31) == 0) {
-            atomicAdd(&bc.c[GV_C_STEPS], static_cast<unsigned long long>(wst));
-            if (wg) atomicAdd(&bc.c[GV_C_STEPS_G], static_cast<unsigned long long>(wg));
-            if (we) atomicAdd(&bc.c[GV_C_STEPS_EM], static_cast<unsigned long long>(we));
-            if (wst - wg - we) atomicAdd(&bc.c[GV_C_STEPS_EP], static_cast<unsigned long long>(wst - wg - we));
-            if (wx) atomicAdd(&bc.c[GV_C_DISCRETE], static_cast<unsigned long long>(wx));
-            if (wb) atomicAdd(&bc.c[GV_C_GEOM], static_cast<unsigned long long>(wb));
-          }
-        }
-        if ((tid & 31) == 0 && wiq) atomicAdd(&bc.c[GV_C_LANE_SLOTS], 32ull * wiq);
-      }
-      if (was_alive && !alive) track_ended(S, t.ev);
-      const bool hand = alive && proc >= 0;
-      emit_requests(S, t, hand, proc, kstep, u);
-      alive = alive && !hand;  // the interaction kernel owns it now
+      uint32_t kstep;
+      R u2 = R(0), u3 = R(0);
+      Run<R> run;
+      const int key = run_round<R, true, true, true>(V, S, t, alive, S->along_steps_g, S->along_steps, kstep, u2, u3, run,
+                                                     static_cast<Pending<R> *>(nullptr));
+      count_round(row, run, t.type, key >= 0 && key != kKeyRest);
+      if (book && was_alive && !alive && key < 0 && book_live(S, t.ev, -1) == 1u) event_closed(S, t.ev);
+      emit_requests(S, t, key, kstep, u2, u3);
+      if (key >= 0) alive = false;  // the interaction kernel owns it now
     }
-    push_survivor(S, out, t, alive);
+    push_track(S, out, t, alive);
   }
   __syncthreads();
-  if (tid < 16 && bc.c[tid]) atomicAdd(&ctl->counters[tid], bc.c[tid]);
+  if (tid < 16) {
+    unsigned long long v = 0ull;
+    for (unsigned w = 0; w < blockDim.x / 32; ++w) v += s_wc[w][tid];
+    if (v) atomicAdd(&ctl->counters[tid], v);
+  }
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__restrict__ S, int parity) {
   __shared__ View<R> sV;
-  __shared__ BlockCnt bc;
+  __shared__ WarpCnt s_wc[8];
   __shared__ unsigned s_kend[kNReqKey], s_kn[kNReqKey];
   __shared__ int s_last;
   Ctl *ctl = S->ctl;
@@ -1424,10 +1551,12 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
       s_kend[k] = acc;
     }
   }
-  if (tid < 16) bc.c[tid] = 0;
+  unsigned long long *const row = s_wc[tid >> 5];
+  if (lane < 16) row[lane] = 0ull;
   __syncthreads();
   const View<R> &V = sV;
   const int out = parity ^ 1;
+  const bool book = ctl->book != 0;
   for (;;) {
     unsigned chunk = 0;
     if (lane == 0) chunk = atomicAdd(&ctl->claim_b, 1u);
@@ -1436,17 +1565,17 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
     int k = 0;
     while (chunk >= s_kend[k]) ++k;
     const unsigned pos = (chunk - (k ? s_kend[k - 1] : 0u)) * 32u + lane;
-    const bool has = pos < s_kn[k];
-    const int ty = k / 3, proc = k - 3 * ty;
     Trk<R> t;
+    t.type = 0;
     Kids<R> kids;
     kids.n = 0;
-    Parent par;
+    Parent par = {0.0, 0.0, 0.0, 0ull, 0u, 0};
     uint32_t kk = 0;
+    int np = 0, na = 0;
+    unsigned was = 0u;
     bool alive = false;
-    if (has) {
+    if (pos < s_kn[k]) {
       const GReq<R> q = S->req[S->keyidx[static_cast<size_t>(k) * S->req_cap + pos]];
-      R uu[8] = {R(0), R(0), q.u[0], q.u[1], q.u[2], q.u[3], q.u[4], q.u[5]};
       R d[3] = {q.d0, q.d1, q.d2};
       R e = q.E;
       t.x = q.x; t.y = q.y; t.z = q.z;
@@ -1454,28 +1583,30 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
       t.ev = q.ev;
       t.sub = q.sf & 0xffff;
       t.flags = q.sf >> 16;
-      t.type = ty;
+      t.type = k / 3;
       kk = q.kk;
       t.step = kk + 1;
       t.nlam = R(-1);
-      const int r = final_state(V, S, &bc, ty, proc, e, d, uu, kids, t.ev, t.sub, t.x, t.y, q.id, q.kk);
+      const int r = final_state<R>(V, S, k, e, d, q.u2, q.u3, kids, t.ev, t.sub, t.x, t.y, q.id, q.kk, np, na);
       t.E = e;
       t.u = d[0]; t.v = d[1]; t.w = d[2];
       if (r >= 0) t.flags |= kFlagInteracted;
       alive = r != 0;
-      par = parent_of(t);
-    } else {
-      par.x = par.y = par.z = 0.0;
-      par.id = 0;
-      par.ev = 0;
-      par.sub = 0;
+      par = Parent{t.x, t.y, t.z, t.id, t.ev, t.sub};
+      if (book) was = book_live(S, t.ev, kids.n - (alive ? 0 : 1));
     }
-    push_kids(S, out, par, kids, kk, &bc);
-    if (has && !alive) track_ended(S, t.ev);
-    push_survivor(S, out, t, alive);
+    wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
+    wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
+    push_kids<R>(S, out, par, kids, kk, row);
+    push_track(S, out, t, alive);
+    if (was == 1u) event_closed(S, t.ev);
   }
   __syncthreads();
-  if (tid < 16 && bc.c[tid]) atomicAdd(&ctl->counters[tid], bc.c[tid]);
+  if (tid < 16) {
+    unsigned long long v = 0ull;
+    for (unsigned w = 0; w < blockDim.x / 32; ++w) v += s_wc[w][tid];
+    if (v) atomicAdd(&ctl->counters[tid], v);
+  }
   __syncthreads();
   if (tid == 0) {
     __threadfence();
@@ -1541,7 +1672,7 @@ struct Ctx {
     bool timed_loop = false; // kernel time = t0 .. t1 of the one graph launch
   } pend;
   ModelMeta meta[kNModel];
-  size_t xs_bytes = 0, zb_bytes = 0, smem_bytes = 0, req_off = 0, bins_bytes = 0, smax_bytes = 0, smax_off = 0;
+  size_t xs_bytes = 0, zb_bytes = 0, smem_bytes = 0, req_off = 0, bins_bytes = 0, smax_bytes = 0, smax_off = 0, thick_off = 0;
   size_t lk_off = 0;
   int grid = 0, grid_b = 0;
   // split pipeline: interaction requests and their per-key index lists
@@ -1605,37 +1736,6 @@ int validate_cfg(const gv_config &c) {
   if (c.blocking < 0 || c.blocking > 1) return GV_ERR_BAD_ARG;
   if (c.pipeline < 0 || c.pipeline > 1 || (c.pipeline == 1 && c.scoring != 0)) return GV_ERR_BAD_ARG;
   return GV_OK;
-}
-
-template <typename R> size_t queue_bytes(long long cap) { return static_cast<size_t>(cap) * track_bytes<R>(); }
-
-template <typename R> Queue<R> carve(unsigned char *&p, long long cap) {
-  Queue<R> q;
-  auto take = [&](size_t n) {
-    unsigned char *r = p;
-    p += (n + 255) / 256 * 256;
-    return r;
-  };
-  q.x = reinterpret_cast<double *>(take(cap * sizeof(double)));
-  q.y = reinterpret_cast<double *>(take(cap * sizeof(double)));
-  q.z = reinterpret_cast<double *>(take(cap * sizeof(double)));
-  q.u = reinterpret_cast<R *>(take(cap * sizeof(R)));
-  q.v = reinterpret_cast<R *>(take(cap * sizeof(R)));
-  q.w = reinterpret_cast<R *>(take(cap * sizeof(R)));
-  q.E = reinterpret_cast<R *>(take(cap * sizeof(R)));
-  q.nlam = reinterpret_cast<R *>(take(cap * sizeof(R)));
-  q.id = reinterpret_cast<unsigned long long *>(take(cap * sizeof(unsigned long long)));
-  q.ev = reinterpret_cast<unsigned *>(take(cap * sizeof(unsigned)));
-  q.step = reinterpret_cast<unsigned *>(take(cap * sizeof(unsigned)));
-  q.sf = reinterpret_cast<int *>(take(cap * sizeof(int)));
-  return q;
-}
-
-template <typename R> size_t carve_bytes(long long cap) {
-  size_t s = 0;
-  const size_t sizes[12] = {8, 8, 8, sizeof(R), sizeof(R), sizeof(R), sizeof(R), sizeof(R), 8, 4, 4, 4};
-  for (size_t z : sizes) s += (cap * z + 255) / 256 * 256;
-  return s;
 }
 
 template <typename R> int upload_tables(Ctx *c) {
@@ -1716,6 +1816,7 @@ template <typename R> View<R> make_view(const Ctx *c) {
   v.smat = c->d_smat;
   v.bins = reinterpret_cast<const AliasBin<R> *>(c->d_bins);
   v.smax = reinterpret_cast<const R *>(c->d_smax);
+  v.thick = nullptr;  // staged by the step kernels
   v.status = nullptr;  // unit kernels: no status word
   for (int m = 0; m < kNModel; ++m) v.meta[m] = c->meta[m];
   v.geo.nsub = c->nsub;
@@ -1851,7 +1952,7 @@ template <typename R> int prepare_device(Ctx *c) {
   rc = setup_l2_window(c);
   if (rc) return rc;
   const long long cap = c->cfg.stack_capacity;
-  const size_t per = carve_bytes<R>(cap);
+  const size_t per = TrackLayout<R>::queue_bytes(cap);
   if (cudaMalloc(&c->d_queues, per * 6) != cudaSuccess) return GV_ERR_OOM;
   CK(cudaMalloc(&c->d_ctl, sizeof(Ctl)));
   CK(cudaMemset(c->d_ctl, 0, sizeof(Ctl)));
@@ -1859,7 +1960,8 @@ template <typename R> int prepare_device(Ctx *c) {
   CK(cudaMallocHost(&c->h_ctl, sizeof(Ctl)));
   c->zb_bytes = ((c->nsub + 1) * sizeof(double) + 15) / 16 * 16;
   c->smax_off = c->xs_bytes + c->zb_bytes + kInvNodeBytes + (c->nsub + 15) / 16 * 16;
-  c->req_off = c->smax_off + c->smax_bytes;
+  c->thick_off = c->smax_off + c->smax_bytes;
+  c->req_off = (c->thick_off + c->nsub * sizeof(R) + 31) / 32 * 32;
   if (c->cfg.pipeline) {
     const size_t rc_ = static_cast<size_t>(cap);
     if (cudaMalloc(&c->d_req, rc_ * sizeof(GReq<R>)) != cudaSuccess ||
@@ -1877,9 +1979,10 @@ template <typename R> int prepare_device(Ctx *c) {
     c->grid_b = c->sm_count * occ_b;
     return GV_OK;
   }
-  c->smem_bytes = c->req_off + (c->cfg.process_sort ? sizeof(IReq<R>) * c->cfg.block_size : 0);
-  c->lk_off = (c->smem_bytes + 15) / 16 * 16;
-  if (c->cfg.process_sort && c->cfg.local_stack) c->smem_bytes = c->lk_off + sizeof(LKid<R>) * c->cfg.block_size;
+  c->smem_bytes = c->req_off + (c->cfg.process_sort ? static_cast<size_t>(ReqStore<R>::kBytes) * c->cfg.block_size : 0);
+  c->lk_off = (c->smem_bytes + 31) / 32 * 32;
+  if (c->cfg.process_sort && c->cfg.local_stack)
+    c->smem_bytes = c->lk_off + static_cast<size_t>(LocalStack<R>::kBytes) * c->cfg.block_size;
   const void *kern = reinterpret_cast<const void *>(pick_step_kernel<R>(c));
   CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
   int occ = 0;
@@ -1893,9 +1996,9 @@ template <typename R> DevState<R> make_state(Ctx *c) {
   DevState<R> s;
   std::memset(&s, 0, sizeof(s));
   s.view = make_view<R>(c);
-  unsigned char *p = static_cast<unsigned char *>(c->d_queues);
-  for (int par = 0; par < 2; ++par)
-    for (int q = 0; q < 3; ++q) s.q[par][q] = carve<R>(p, c->cfg.stack_capacity);
+  s.qmem = static_cast<unsigned char *>(c->d_queues);
+  s.q_bytes = TrackLayout<R>::queue_bytes(c->cfg.stack_capacity);
+  s.q_part = TrackLayout<R>::part_bytes(c->cfg.stack_capacity);
   s.capacity = static_cast<unsigned long long>(c->cfg.stack_capacity);
   s.ctl = c->d_ctl;
   s.view.status = &c->d_ctl->status;  // device address; checks of the checking build
@@ -1923,6 +2026,7 @@ template <typename R> DevState<R> make_state(Ctx *c) {
   s.zb_bytes = static_cast<unsigned>(c->zb_bytes);
   s.smem_req_off = static_cast<unsigned>(c->req_off);
   s.smax_off = static_cast<unsigned>(c->smax_off);
+  s.thick_off = static_cast<unsigned>(c->thick_off);
   s.smem_lk_off = static_cast<unsigned>(c->lk_off);
   s.local_stack = c->cfg.local_stack;
   s.smax_bytes = static_cast<unsigned>(c->smax_bytes);
@@ -2492,7 +2596,7 @@ constexpr size_t kStaticQueueBytes = 6 * static_cast<size_t>(kStaticCap) * track
 constexpr size_t kStaticBytes = kStaticQueueOff + kStaticQueueBytes;  // 25,440,256 bytes
 static_assert(sizeof(Ctl) <= kStaticStateOff - kStaticCtlOff, "control block does not fit");
 static_assert(sizeof(DevState<float>) <= kStaticEvliveOff - kStaticStateOff, "state does not fit");
-static_assert(kStaticCap % 64 == 0, "queue arrays must stay 256-byte aligned");
+static_assert(kStaticCap % 16 == 0, "queue parts must stay 256-byte aligned");
 }  // namespace
 
 static __device__ __align__(256) unsigned char g_gv_static_scratch[kStaticBytes];
@@ -2511,31 +2615,6 @@ int static_scratch(unsigned char **base) {
   }
   *base = static_cast<unsigned char *>(p);
   return GV_OK;
-}
-
-// carve the queues of the scratch array exactly as carve() does for the
-// context's own allocation (every array a multiple of 256 bytes long)
-Queue<float> carve_static(unsigned char *&p) {
-  Queue<float> q;
-  auto take = [&](size_t n) {
-    unsigned char *r = p;
-    p += n;
-    return r;
-  };
-  const size_t C = static_cast<size_t>(kStaticCap);
-  q.x = reinterpret_cast<double *>(take(C * 8));
-  q.y = reinterpret_cast<double *>(take(C * 8));
-  q.z = reinterpret_cast<double *>(take(C * 8));
-  q.u = reinterpret_cast<float *>(take(C * 4));
-  q.v = reinterpret_cast<float *>(take(C * 4));
-  q.w = reinterpret_cast<float *>(take(C * 4));
-  q.E = reinterpret_cast<float *>(take(C * 4));
-  q.nlam = reinterpret_cast<float *>(take(C * 4));
-  q.id = reinterpret_cast<unsigned long long *>(take(C * 8));
-  q.ev = reinterpret_cast<unsigned *>(take(C * 4));
-  q.step = reinterpret_cast<unsigned *>(take(C * 4));
-  q.sf = reinterpret_cast<int *>(take(C * 4));
-  return q;
 }
 
 // the state record travels as a kernel argument, so no staging copy is needed
@@ -2586,9 +2665,9 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
       cudaMemsetAsync(base + kStaticEvliveOff, 0, sizeof(unsigned) * n_events, st) != cudaSuccess)
     return GV_ERR_CUDA;
   DevState<float> s = make_state<float>(c);
-  unsigned char *qp = base + kStaticQueueOff;
-  for (int par = 0; par < 2; ++par)
-    for (int q = 0; q < 3; ++q) s.q[par][q] = carve_static(qp);
+  s.qmem = base + kStaticQueueOff;
+  s.q_bytes = TrackLayout<float>::queue_bytes(kStaticCap);
+  s.q_part = TrackLayout<float>::part_bytes(kStaticCap);
   s.capacity = static_cast<unsigned long long>(kStaticCap);
   s.ctl = reinterpret_cast<Ctl *>(base + kStaticCtlOff);
   s.view.status = &s.ctl->status;
