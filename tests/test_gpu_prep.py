@@ -1,0 +1,68 @@
+"""What surrounds the generations: the prefix sums of the primaries' budgets
+(blocks of 256 primaries each, up to 304 blocks and then longer ranges), and
+tallies accumulated in the caller's buffers or copied to them."""
+import numpy as np
+import pytest
+
+from paper_2005_00949_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gvmod():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    return gv
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 304 * 256, 304 * 256 + 1, 100_003])
+def test_budget_sums_admit_every_primary(gvmod, n):
+    """Uneven photons through a queue that holds a few hundred of them at a
+    time: the automatic cap reads the budget sums at every generation, admits
+    all primaries and never overflows, and the results are those of a queue
+    that holds all at once."""
+    wl = W.photon_slab(n, 0.3)
+    wl.primaries["E"] = 0.05 + 0.9 * np.random.default_rng(n).random(n)
+    runs = []
+    for cap in (1 << 16, 1 << 24):
+        ctx = gvmod.Context(wl, gvmod.gv_default_config(stack_capacity=cap, per_event_counts=1))
+        runs.append(ctx.transport(per_event=True))
+        ctx.close()
+        assert runs[-1]["status"] == 0
+        assert runs[-1]["counters"]["live_peak"] <= cap
+    assert np.array_equal(runs[0]["counts"][:, :11], runs[1]["counts"][:, :11])
+    assert runs[0]["counters"]["tracks_gamma"] == n
+    if n > 2048:  # 64 budgeted tracks each and a little: about a thousand photons in flight
+        assert runs[0]["counters"]["live_peak"] <= 1024
+    total = runs[0]["edep"].sum(1) + runs[0]["escape"]
+    assert np.abs(total - wl.primaries["E"]).max() < 1e-6
+
+
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable", "unaligned"])
+def test_tallies_in_place_or_copied(gvmod, where):
+    import torch
+    wl = W.wsi_cells(5, 3000.0)
+    ctx = gvmod.Context(wl, gvmod.gv_default_config(stack_capacity=1 << 18, per_event_counts=1))
+    ref = ctx.transport(per_event=True)
+    shapes = {"edep": (5, ctx.n_subtotal), "escape": (5,), "cell": (50 * 32 * 32,), "counts": (5, gvmod.NCOUNT)}
+    buf = {}
+    for k, shape in shapes.items():
+        dtype = torch.int64 if k == "counts" else torch.float64
+        if where == "unaligned":  # 4 bytes off: copied, not accumulated in place
+            raw = torch.full((8 * int(np.prod(shape)) + 8,), 7, dtype=torch.uint8, device="cuda")
+            buf[k] = raw[4:-4]
+        else:
+            buf[k] = torch.full(shape, 7, dtype=dtype, device="cuda" if where == "device" else "cpu")
+            if where == "pinned":
+                buf[k] = buf[k].pin_memory()
+    for _ in range(2):  # the second call starts from the first one's results
+        ctx.gv_transport(wl.primaries, 5, wl.seed, buf["edep"], buf["cell"], buf["escape"], buf["counts"])
+    torch.cuda.synchronize()
+    got = {k: v.cpu().numpy().copy().view(np.int64 if k == "counts" else np.float64).reshape(shapes[k])
+           for k, v in buf.items()}
+    ctx.close()
+    assert np.array_equal(got["counts"][:, :11], ref["counts"][:, :11])
+    for k in ("edep", "escape", "cell"):  # the order of the FP64 sums
+        assert np.abs(got[k].ravel() - ref[k].ravel()).max() < 1e-9 * 3000.0, k
