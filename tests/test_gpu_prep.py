@@ -1,4 +1,4 @@
-"""What surrounds the generations: the prefix sums of the primaries' budgets
+"""What surrounds the generations (and the sampler entry point): the prefix sums of the primaries' budgets
 (blocks of 256 primaries each, up to 304 blocks and then longer ranges), and
 tallies accumulated in the caller's buffers or copied to them."""
 import numpy as np
@@ -66,3 +66,30 @@ def test_tallies_in_place_or_copied(gvmod, where):
     assert np.array_equal(got["counts"][:, :11], ref["counts"][:, :11])
     for k in ("edep", "escape", "cell"):  # the order of the FP64 sums
         assert np.abs(got[k].ravel() - ref[k].ravel()).max() < 1e-9 * 3000.0, k
+
+
+@pytest.mark.parametrize("model", range(6))
+def test_sampler_kernels_agree_at_their_border(gvmod, model):
+    """From 2^18 samples on the sampling tables are read from shared memory:
+    the same tables and arithmetic in another kernel, so equal up to the
+    rounding of separately compiled FP32 code (a few ulp), except where that
+    decides a table bin (bounded at 1e-4 of the samples)."""
+    import torch
+    border = 1 << 18
+    wl = W.pbps_electrons(1)
+    ctx = gvmod.Context(wl, gvmod.gv_default_config(stack_capacity=1 << 12))
+    n = border + 77
+    lo = [0.01, 2.0, 1.5, 3.0, 2.0, 0.01][model]
+    E = torch.from_numpy(lo * 10.0 ** (4.0 * np.random.default_rng(model).random(n))).cuda()
+    outs = []
+    for m in (border - 1, border, n):
+        out = torch.full((n, 3), -7.0, dtype=torch.float64, device="cuda")
+        ctx.gv_unit_sample(model, 0, E[:m], 99, out)
+        outs.append(out.cpu().numpy())
+        assert (outs[-1][m:] == -7.0).all()
+        assert (outs[-1][:m, 2] == 1.0).all()
+    ctx.close()
+    assert np.array_equal(outs[1][:border], outs[2][:border])
+    a, b = outs[0][:border - 1], outs[1][:border - 1]
+    off = np.abs(a - b) > 1e-6 * np.maximum(np.abs(a), 1e-30)
+    assert off.any(axis=1).mean() < 1e-4
