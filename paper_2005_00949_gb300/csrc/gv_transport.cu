@@ -457,7 +457,7 @@ __device__ __forceinline__ int run_round(const View<R> &V, const DevState<R> *S,
 // deposit.  Returns 1 if the particle survives, 0 if it ended, -1 if the
 // process was kinematically closed at the post-step energy (nothing
 // changes).  np, na: pairs and annihilations made.
-template <typename R, bool OPTS = true, bool EXT = true>
+template <typename R, bool OPTS = true, bool EXT = true, bool ALT = false>
 __device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *S, int key, R &E, R d[3], R u2, R u3,
                                            Kids<R> &kids, unsigned ev, int sub, double x, double y,
                                            unsigned long long id, uint32_t kk, int &np, int &na,
@@ -473,7 +473,7 @@ __device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *
     R local;
     const RngKey g = {static_cast<uint32_t>(id), static_cast<uint32_t>(id >> 32), kk, S->seed_lo ^ (ev + S->ev_base),
                       S->seed_hi};
-    r = interact<R, OPTS>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na);
+    r = interact<R, OPTS, ALT>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na);
     if (r < 0) return -1;
     deposit<R, EXT>(V, S, ev, sub, x, y, local, pd);
   }
@@ -1248,7 +1248,7 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 // 5.39 ms a transport; 1000 x 1 GeV: 1.41 -> 1.13 ms; 300 x 10 GeV in FP64:
 // 13.4 -> 10.8 ms (its arithmetic sits on the FP64 pipe); 2000 x 100 GeV in
 // W/Si with cells: 95.6 -> 65.5 ms.
-template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT>
+template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT, bool ALT = !SORT>
 __global__ void GV_STEP_BOUNDS
     step_kernel(int parity) {
   const DevState<R> *__restrict__ S = tstate<R>();
@@ -1408,7 +1408,7 @@ __global__ void GV_STEP_BOUNDS
         int np = 0, na = 0, change = own_end ? -1 : 0;
         if (key >= 0) {
           R d[3] = {t.u, t.v, t.w};
-          const int r = final_state<R, OPTS, EXT>(V, S, key, t.E, d, u2, u3, kids, t.ev, t.sub, t.x, t.y, t.id, kstep, np,
+          const int r = final_state<R, OPTS, EXT, ALT>(V, S, key, t.E, d, u2, u3, kids, t.ev, t.sub, t.x, t.y, t.id, kstep, np,
                                                   na, pd);
           if (r >= 0) {
             t.u = d[0]; t.v = d[1]; t.w = d[2];
@@ -1496,7 +1496,7 @@ __global__ void GV_STEP_BOUNDS
           pk = g.y;
           R d[3] = {dE.x, dE.y, dE.z};
           R e = dE.w;
-          const int r = final_state<R, OPTS, EXT>(V, S, static_cast<int>(g.w), e, d, req.u2(tid), req.u3(tid), kb, par.ev,
+          const int r = final_state<R, OPTS, EXT, ALT>(V, S, static_cast<int>(g.w), e, d, req.u2(tid), req.u3(tid), kb, par.ev,
                                                   par.sub, par.x, par.y, par.id, pk, np, na);
           req.dir(tid) = V4<R>{d[0], d[1], d[2], e};
           req.ret(tid) = r;
@@ -2837,13 +2837,20 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
   unsigned char *base = nullptr;
   int rc = static_scratch(&base);
   if (rc) return rc;
-  const size_t smem = c->req_off;  // tables and geometry; the non-basketizing kernel
-  if (cudaFuncSetAttribute(step_kernel<float, false, false, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  // the basketizing kernel (with the arithmetic of the one without, which this
+  // call ran before: the same showers at half the time)
+  bool opts = (c->cuts.process_mask & (GV_P_MSC | GV_P_INTEGRAL)) != 0;
+  for (int m = 0; m < kNModel; ++m) opts = opts || c->cuts.reject_min_MeV[m] < 1e30;
+  const StepFn<float> step = opts ? step_kernel<float, true, false, false, true, false, true>
+                                  : step_kernel<float, true, false, false, false, false, true>;
+  const int block = c->cfg.block_size;
+  const size_t lk_off = (c->req_off + static_cast<size_t>(ReqStore<float>::kBytes) * block + 31) / 32 * 32;
+  const size_t smem = lk_off + static_cast<size_t>(LocalStack<float>::kBytes) * block;
+  if (cudaFuncSetAttribute(reinterpret_cast<const void *>(step), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem)) != cudaSuccess)
     return GV_ERR_CUDA;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, step_kernel<float, false, false, false, true, true>, c->cfg.block_size, smem) !=
-          cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, reinterpret_cast<const void *>(step), block, smem) != cudaSuccess ||
       occ < 1)
     return GV_ERR_CUDA;
   const int grid = c->sm_count * std::min(occ, c->cfg.blocks_per_sm);
@@ -2860,9 +2867,11 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
   s.ctl = reinterpret_cast<Ctl *>(base + kStaticCtlOff);
   s.view.status = &s.ctl->status;
   s.mode = GV_BATCHED;
-  s.chunk = c->cfg.block_size;  // the non-basketizing kernel, one claim per block
-  s.adaptive_chunk = 0;
-  s.claim_chunks = 0;
+  s.chunk = block;
+  s.adaptive_chunk = 1;
+  s.grid = grid;
+  s.pipeline = 0;
+  s.smem_lk_off = static_cast<unsigned>(lk_off);
   s.low_water = static_cast<unsigned long long>(kStaticCap / 4);
   s.batch = std::min<unsigned long long>(s.batch, 64);
   s.max_in_flight = -1;  // automatic: capacity / (0.15 per MeV of the most energetic primary + 64)
@@ -2886,17 +2895,34 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
     prim_emax_kernel<float><<<static_cast<int>(std::min<long long>((n + 255) / 256, 4 * c->sm_count)), 256, 0, st>>>(S);
   init_kernel<float><<<1, 1, 0, st>>>(S);
   if (cudaGetLastError() != cudaSuccess) return GV_ERR_CUDA;
-  int between = 1;
-  for (;;) {
-    for (int i = 0; i < 2 * between; ++i)
-      step_kernel<float, false, false, false, true, true><<<grid, c->cfg.block_size, smem, st>>>(i & 1);
-    if (cudaGetLastError() != cudaSuccess) return GV_ERR_CUDA;
+  // Generations go out in batches, and the next batch before the host has seen
+  // whether the last one ended the transport: the GPU does not wait for the
+  // host, and at most two batches of generations return at once.
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(block);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  lc.attrs = attr;
+  constexpr int kBatch = 12;  // even: a batch starts at parity 0
+  const cudaEvent_t seen[2] = {c->ev_in, c->ev_out};
+  for (int batch = 0;; ++batch) {
+    for (int i = 0; i < kBatch; ++i) {
+      lc.numAttrs = (c->cfg.pdl && i > 0) ? 1 : 0;
+      const int parity = i & 1;
+      if (cudaLaunchKernelEx(&lc, step, parity) != cudaSuccess) return GV_ERR_CUDA;
+    }
     if (cudaMemcpyAsync(c->h_ctl, s.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+        cudaEventRecord(seen[batch & 1], st) != cudaSuccess)
       return GV_ERR_CUDA;
-    if (c->h_ctl->done) break;
-    between = std::min(between * 2, 32);
+    if (batch == 0) continue;
+    if (cudaEventSynchronize(seen[(batch - 1) & 1]) != cudaSuccess) return GV_ERR_CUDA;
+    if (*const_cast<volatile int *>(&c->h_ctl->done)) break;  // final once set, whichever batch it came with
   }
+  if (cudaStreamSynchronize(st) != cudaSuccess) return GV_ERR_CUDA;
   for (int i = 0; i < 16; ++i) counters[i] = c->h_ctl->counters[i];
   counters[GV_C_GENERATIONS] = c->h_ctl->gen;
   counters[15] = c->h_ctl->live_peak;
