@@ -61,34 +61,42 @@ template <typename R> struct alignas(16) GReq {
 constexpr int kNReqKey = 9;
 constexpr int kKeyRest = 1 * 3 + 2;
 
+// The plan of a generation, one 64-byte record: a block reads all of it in
+// one round trip to L2 when the generation before has completed.
+struct alignas(64) Plan {
+  int done;                  // the transport has ended: nothing is planned
+  int K;                     // rounds per claimed track
+  unsigned B;                // tracks per block claim
+  int book;                  // events are counted live (primaries are still waiting on the in-flight cap)
+  unsigned end[4];           // cumulative chunk counts in claim order: e+, e-, gamma, primaries
+  unsigned n_in[3];          // tracks in the input queues (within the capacity)
+  unsigned prim_begin, prim_count;
+  unsigned pad[3];
+};
+
 // Generation control block.  The last block of every generation writes the
 // plan of the next one; kernels only read it.
 struct Ctl {
   ClaimSlot claims[kNClaim];
   FillSlot cnt[2][3];        // queue fill per buffer parity and type
   ClaimSlot claim;           // chunk claim counter of the block claims
+  Plan plan;
   unsigned prim_next;        // primaries handed out so far
-  unsigned prim_begin, prim_count;
-  unsigned chunk_end[4];     // cumulative chunk counts in claim order: e+, e-, gamma, primaries
   unsigned blocks_done;
-  int K;                     // steps per claimed track this generation
-  unsigned chunk_B;          // tracks per block claim this generation
   int status;
-  int done;
-  int book;                  // events are counted live (primaries are still waiting on the in-flight cap)
   unsigned ev_started, ev_done;  // events whose live-track count left / returned to zero
   unsigned max_in_flight;        // refill cap of this call (0: none)
   unsigned emax_bits;            // largest primary energy (FP32 bits), for the automatic cap
   unsigned long long gen;
   unsigned long long loop_iter;  // bodies of the device-side generation loop run so far
   unsigned long long live_peak;
+  unsigned long long cost_started, cost_done;  // automatic cap: track budget taken by / returned from events
   unsigned long long counters[16];
   // split pipeline: requests of this generation, per key, and the claim /
   // completion counters of the interaction kernel
   unsigned req_n;
   unsigned key_n[kNReqKey];
   unsigned claim_b, blocks_done_b;
-  unsigned long long cost_started, cost_done;  // automatic cap: track budget taken by / returned from events
 };
 
 template <typename R> struct DevState {

@@ -964,17 +964,25 @@ __device__ __forceinline__ int claim_queue(int seg) { return seg < 3 ? 2 - seg :
 
 template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   Ctl *c = S->ctl;
+  // everything the plan depends on, in one round trip
+  const unsigned cap = static_cast<unsigned>(S->capacity);
   const unsigned n0 = c->cnt[pn][0].n, n1 = c->cnt[pn][1].n, n2 = c->cnt[pn][2].n;
+  const unsigned next = c->prim_next, max_in_flight = c->max_in_flight;
+  const unsigned ev_started = c->ev_started, ev_done = c->ev_done;
+  unsigned long long cost_started = c->cost_started, cost_done = c->cost_done;
+  const unsigned long long live_peak = c->live_peak;
+  unsigned long long gen = c->gen;
+  int status = c->status;
   const unsigned long long live = static_cast<unsigned long long>(n0) + n1 + n2;
-  const unsigned rem = S->n_prim - c->prim_next;
+  const unsigned rem = S->n_prim - next;
   unsigned inj = 0;
-  if (c->status == 0 && rem > 0) {
+  if (status == 0 && rem > 0) {
     if (S->mode == GV_ONE_EVENT_PER_LAUNCH) {
       if (live == 0) {
-        const unsigned first = S->order ? S->order[c->prim_next] : c->prim_next;
+        const unsigned first = S->order ? S->order[next] : next;
         const unsigned ev = S->prim[first].event;
         while (inj < rem) {
-          const unsigned i = c->prim_next + inj;
+          const unsigned i = next + inj;
           const unsigned pi = S->order ? S->order[i] : i;
           if (S->prim[pi].event != ev) break;
           ++inj;
@@ -982,16 +990,16 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
       }
     } else if (live < S->low_water || live == 0) {
       inj = rem < S->batch ? rem : static_cast<unsigned>(S->batch);
-      if (c->max_in_flight) {  // events in flight (Sec. 2.1.1): started and not yet finished
-        const unsigned fl = c->ev_started - c->ev_done;
-        const unsigned room = c->max_in_flight > fl ? c->max_in_flight - fl : 0u;
+      if (max_in_flight) {  // events in flight (Sec. 2.1.1): started and not yet finished
+        const unsigned fl = ev_started - ev_done;
+        const unsigned room = max_in_flight > fl ? max_in_flight - fl : 0u;
         inj = inj < room ? inj : room;
       }
       if (S->pcost && inj > 0) {  // automatic cap: the budgets of the events in flight fit the capacity
-        if (live == 0) c->cost_done = c->cost_started;  // nothing alive: every event has closed
-        const unsigned long long held = c->cost_started > c->cost_done ? c->cost_started - c->cost_done : 0ull;
+        if (live == 0) c->cost_done = cost_done = cost_started;  // nothing alive: every event has closed
+        const unsigned long long held = cost_started > cost_done ? cost_started - cost_done : 0ull;
         const unsigned long long room = S->capacity > held ? S->capacity - held : 0ull;
-        const unsigned long long *pc = S->pcost + c->prim_next;
+        const unsigned long long *pc = S->pcost + next;
         const unsigned long long base = pc[0];
         if (pc[inj] - base > room) {  // the longest run of the next primaries that fits
           unsigned lo = 0, hi = inj;  // budget(lo) <= room < budget(hi)
@@ -1003,16 +1011,19 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
           inj = lo;
         }
         if (inj == 0 && live == 0) inj = 1;  // one primary at least when nothing is alive
-        c->cost_started += pc[inj] - base;
+        c->cost_started = cost_started + (pc[inj] - base);
       }
     }
   }
-  c->prim_begin = c->prim_next;
-  c->prim_count = inj;
-  c->prim_next += inj;
+  const unsigned long long tot = live + inj;
+  const bool last = next + inj == S->n_prim;
+  Plan p;
+  p.prim_begin = next;
+  p.prim_count = inj;
+  c->prim_next = next + inj;
   // the events' live tracks are asked for only by the in-flight cap, and that
   // only while primaries wait
-  c->book = S->mode == GV_BATCHED && c->prim_next < S->n_prim && (c->max_in_flight || S->pcost);
+  p.book = S->mode == GV_BATCHED && !last && (max_in_flight || S->pcost);
   unsigned B = static_cast<unsigned>(S->chunk);
   // With fewer live tracks than the grid has lanes (the first generations of
   // a shower and its tail), a block claims fewer tracks (a multiple of 32)
@@ -1020,20 +1031,22 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   // fewer warps to wait for at its barriers and its idle lanes left to the
   // secondaries of its block stack.
   if (S->adaptive_chunk) {
-    const unsigned long long tot = live + inj;
     const unsigned long long per = (tot + S->grid - 1) / S->grid;
     if (per < B) B = per <= 32 ? 32u : static_cast<unsigned>((per + 31) / 32 * 32);
   }
-  c->chunk_B = B;
-  c->chunk_end[0] = (n2 + B - 1) / B;  // segments in claim_queue order
-  c->chunk_end[1] = c->chunk_end[0] + (n1 + B - 1) / B;
-  c->chunk_end[2] = c->chunk_end[1] + (n0 + B - 1) / B;
-  c->chunk_end[3] = c->chunk_end[2] + (inj + B - 1) / B;
+  p.B = B;
+  p.end[0] = (n2 + B - 1) / B;  // segments in claim_queue order
+  p.end[1] = p.end[0] + (n1 + B - 1) / B;
+  p.end[2] = p.end[1] + (n0 + B - 1) / B;
+  p.end[3] = p.end[2] + (inj + B - 1) / B;
+  p.n_in[0] = min(n0, cap);
+  p.n_in[1] = min(n1, cap);
+  p.n_in[2] = min(n2, cap);
   // long claims (K_tail rounds) once every primary is injected and few
   // tracks are live: in the tail, and at the start of a batch injected at
   // once, where the block stack keeps a claim's secondaries stepping in the
   // block (one-round claims there measured slower on small batches)
-  c->K = (c->prim_next == S->n_prim && live + inj < S->tail_threshold) ? S->K_tail : S->K_bulk;
+  p.K = (last && tot < S->tail_threshold) ? S->K_tail : S->K_bulk;
   for (int q = 0; q < 3; ++q) c->cnt[pn ^ 1][q].n = 0;
   c->claim.n = 0;
   for (int r = 0; r < kNClaim; ++r) c->claims[r].n = 0;
@@ -1042,12 +1055,13 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   for (int k = 0; k < kNReqKey; ++k) c->key_n[k] = 0;
   c->claim_b = 0;
   c->blocks_done_b = 0;
-  if (live + inj > c->live_peak) c->live_peak = live + inj;
-  if (live + inj > 0) c->gen += 1;
-  if (c->gen > S->max_gen && c->status == 0) c->status = GV_ERR_TIMEOUT;
-  c->done = (c->status != 0) || (live == 0 && inj == 0 && c->prim_next == S->n_prim);
-  if (c->done) c->chunk_end[0] = c->chunk_end[1] = c->chunk_end[2] = c->chunk_end[3] = 0;
-  c->counters[GV_C_GENERATIONS] = c->gen;
+  if (tot > live_peak) c->live_peak = tot;
+  if (tot > 0) c->gen = ++gen;
+  if (gen > S->max_gen && status == 0) c->status = status = GV_ERR_TIMEOUT;
+  p.done = (status != 0) || (tot == 0 && last);
+  if (p.done) p.end[0] = p.end[1] = p.end[2] = p.end[3] = 0;
+  p.pad[0] = p.pad[1] = p.pad[2] = 0;
+  c->plan = p;
 }
 
 // The control block of a transport that starts, and the plan of its first
@@ -1058,7 +1072,7 @@ template <typename R> __device__ void start_control(const DevState<R> *S) {
     for (int q = 0; q < 3; ++q) c->cnt[i][q].n = 0;
   c->prim_next = 0;
   c->status = 0;
-  c->done = 0;
+  c->plan.done = 0;
   c->gen = 0;
   c->loop_iter = 0;
   c->live_peak = 0;
@@ -1213,6 +1227,15 @@ template <typename R> __global__ void prim_emax_kernel(const DevState<R> *S) {
 __constant__ DevState<float> c_state_f;
 __constant__ DevState<double> c_state_d;
 template <typename R> __device__ __forceinline__ const DevState<R> *tstate();
+
+// Whether the calling thread's block is the last of the grid to finish; what
+// every block wrote before is then visible to it (each block's other threads
+// reach the counter through a block barrier).
+__device__ __forceinline__ bool block_done(unsigned *counter) {
+  unsigned before;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(counter) : "memory");
+  return before == gridDim.x - 1;
+}
 template <> __device__ __forceinline__ const DevState<float> *tstate<float>() { return &c_state_f; }
 template <> __device__ __forceinline__ const DevState<double> *tstate<double>() { return &c_state_d; }
 
@@ -1255,10 +1278,9 @@ __global__ void GV_STEP_BOUNDS
   extern __shared__ __align__(32) unsigned char smem[];
   __shared__ View<R> sV;
   __shared__ WarpCnt s_wc[GV_MAX_BLOCK / 32];
-  __shared__ unsigned s_chunk, s_end[4], s_pb;
-  __shared__ unsigned s_slice[kNClaim + 1];
-  __shared__ int s_K, s_last, s_book;
-  __shared__ unsigned s_B;
+  __shared__ Plan s_plan;
+  __shared__ unsigned s_chunk;
+  __shared__ unsigned s_slice[SORT ? 1 : kNClaim + 1];
   __shared__ StackCount s_stack;  // the block's secondary stack (local_stack)
   __shared__ unsigned s_key[2][kNKey];  // requests per key of this round and the next
   Ctl *ctl = S->ctl;
@@ -1267,36 +1289,33 @@ __global__ void GV_STEP_BOUNDS
   // start as soon as this one's finish, stage their tables, and wait for
   // this grid (and its plan) to complete before reading the plan.
   asm volatile("griddepcontrol.launch_dependents;");
-  if (ctl->done) return;  // a done flag seen before the wait is final: nothing planned
+  if (ctl->plan.done) return;  // a done flag seen before the wait is final: nothing planned
   unsigned long long *const row = s_wc[tid >> 5];
   if (lane < 16) row[lane] = 0ull;
   if (tid < 2 * kNKey) s_key[tid / kNKey][tid % kNKey] = 0u;
   stage_tables(S, smem, sV);
+  if (tid == 0) {
+    s_stack.used = s_stack.taken[0] = s_stack.taken[1] = 0u;
+    s_chunk = blockIdx.x;  // the first claim is the block's own
+  }
   // the previous generation, and its plan, complete before the plan is read
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (ctl->done) return;  // uniform: nothing planned for this generation
-  const bool block_claims = SORT || S->claim_chunks == 0;
-  if (tid == 0) {
-    for (int i = 0; i < 4; ++i) s_end[i] = ctl->chunk_end[i];
-    for (int r = 0; r <= kNClaim; ++r)
-      s_slice[r] = static_cast<unsigned>((static_cast<unsigned long long>(s_end[3]) * r) / kNClaim);
-    s_pb = ctl->prim_begin;
-    s_K = ctl->K;
-    s_B = ctl->chunk_B;
-    s_book = ctl->book;
-    s_stack.used = s_stack.taken[0] = s_stack.taken[1] = 0u;
-    // the first claim; each later one is issued before the previous claim's survivors go out
-    if (block_claims) s_chunk = atomicAdd(&ctl->claim.n, 1u);
-  }
+  static_assert(sizeof(Plan) == 64, "read in sixteen words");
+  if (tid < 16) reinterpret_cast<unsigned *>(&s_plan)[tid] = reinterpret_cast<const unsigned *>(&ctl->plan)[tid];
   __syncthreads();
+  if (s_plan.done) return;  // uniform: nothing planned for this generation
+  const unsigned *const s_end = s_plan.end;
+  const unsigned s_pb = s_plan.prim_begin;
+  const bool block_claims = SORT || S->claim_chunks == 0;
+  if (!SORT && tid <= kNClaim)
+    s_slice[SORT ? 0 : tid] = static_cast<unsigned>((static_cast<unsigned long long>(s_end[3]) * static_cast<unsigned>(tid)) / kNClaim);
+  if (!SORT) __syncthreads();
   const View<R> &V = sV;
   const int in = parity, out = parity ^ 1;
-  const unsigned cap = static_cast<unsigned>(S->capacity);
-  const unsigned n_prim_gen = ctl->prim_count;
   // With several rounds per claim, the secondaries made in a round stay in
   // the block and fill its idle lanes in the next rounds (local_stack).
-  const bool use_local = SORT && S->local_stack && s_K > 1;
-  const bool book = s_book != 0;
+  const bool use_local = SORT && S->local_stack && s_plan.K > 1;
+  const bool book = s_plan.book != 0;
   LocalStack<R> lstk;
   lstk.e = smem + S->smem_lk_off;
   lstk.count = &s_stack;
@@ -1351,7 +1370,7 @@ __global__ void GV_STEP_BOUNDS
     int qsel = 0;
     while (chunk >= s_end[qsel]) ++qsel;
     {
-      const unsigned csize = block_claims ? s_B : 32u;
+      const unsigned csize = block_claims ? s_plan.B : 32u;
       idx = (chunk - (qsel ? s_end[qsel - 1] : 0u)) * csize + (block_claims ? tid : lane);
       if (block_claims && static_cast<unsigned>(tid) >= csize) idx = 0xffffffffu;
     }
@@ -1361,18 +1380,18 @@ __global__ void GV_STEP_BOUNDS
     t.ev = 0;
     bool alive = false;
     if (qsel < 3) {
-      if (idx < min(ctl->cnt[in][qsel].n, cap)) {
+      if (idx < s_plan.n_in[qsel]) {
         load_track<R>(S, in, qsel, idx, t);
         alive = true;
         GV_CHECK(&ctl->status, t.sub >= 0 && t.sub < V.geo.nsub && t.ev < S->n_events && t.E >= R(0));
       }
     } else {
-      const bool has = idx < n_prim_gen;
+      const bool has = idx < s_plan.prim_count;
       int note = 0;
       if (has) alive = load_primary<R, EXT>(V, S, s_pb + idx, book, t, note);
       count_primaries(row, has, t.type, note);
     }
-    const int K = s_K;
+    const int K = s_plan.K;
     unsigned ended_own = 0u, ended_req = 0u;  // evlive before this lane's last bookings of an end (1: the event closed)
     unsigned ev_req = 0u;
     for (int kk = 0; kk < K; ++kk) {
@@ -1531,7 +1550,7 @@ __global__ void GV_STEP_BOUNDS
     // the next claim's atomic and the event count's are in flight while the
     // survivors are written
     unsigned next_chunk = 0u;
-    if (block_claims && tid == 0) next_chunk = atomicAdd(&ctl->claim.n, 1u);
+    if (block_claims && tid == 0) next_chunk = gridDim.x + atomicAdd(&ctl->claim.n, 1u);
     if (MERGE) warp_flush(S, pend);  // nothing stays pending past a claim
     push_track(S, out, t, alive);
     if (ended_own == 1u) event_closed(S, t.ev);
@@ -1561,16 +1580,7 @@ __global__ void GV_STEP_BOUNDS
     if (v) atomicAdd(&ctl->counters[tid], v);
   }
   __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(&ctl->blocks_done, 1u);
-    s_last = (t == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (s_last && tid == 0) {
-    __threadfence();
-    plan_next(S, out);
-  }
+  if (tid == 0 && block_done(&ctl->blocks_done)) plan_next(S, out);
 }
 
 // ------------------------------------------------------------------ split pipeline
@@ -1633,15 +1643,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? GV_ALONG_MIN_BLOCKS : 2)
   __shared__ unsigned s_chunk;
   Ctl *ctl = S->ctl;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (ctl->done) return;
+  if (ctl->plan.done) return;
   unsigned long long *const row = s_wc[tid >> 5];
   if (lane < 16) row[lane] = 0ull;
   stage_tables(S, smem, sV);
   const View<R> &V = sV;
   const int in = parity, out = parity ^ 1;
-  const unsigned cap = static_cast<unsigned>(S->capacity);
-  const unsigned n_prim_gen = ctl->prim_count, n_chunks = ctl->chunk_end[3];
-  const bool book = ctl->book != 0;
+  const unsigned n_prim_gen = ctl->plan.prim_count, n_chunks = ctl->plan.end[3];
+  const bool book = ctl->plan.book != 0;
   for (;;) {
     if (tid == 0) s_chunk = atomicAdd(&ctl->claim.n, 1u);
     __syncthreads();
@@ -1649,15 +1658,15 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? GV_ALONG_MIN_BLOCKS : 2)
     __syncthreads();
     if (chunk >= n_chunks) break;
     int qsel = 0;
-    while (chunk >= ctl->chunk_end[qsel]) ++qsel;
-    const unsigned idx = (chunk - (qsel ? ctl->chunk_end[qsel - 1] : 0u)) * blockDim.x + tid;
+    while (chunk >= ctl->plan.end[qsel]) ++qsel;
+    const unsigned idx = (chunk - (qsel ? ctl->plan.end[qsel - 1] : 0u)) * blockDim.x + tid;
     qsel = claim_queue(qsel);
     Trk<R> t;
     t.type = 0;
     t.ev = 0;
     bool alive = false;
     if (qsel < 3) {
-      if (idx < min(ctl->cnt[in][qsel].n, cap)) {
+      if (idx < ctl->plan.n_in[qsel]) {
         load_track<R>(S, in, qsel, idx, t);
         alive = true;
         GV_CHECK(&ctl->status, t.sub >= 0 && t.sub < V.geo.nsub && t.ev < S->n_events && t.E >= R(0));
@@ -1665,10 +1674,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? GV_ALONG_MIN_BLOCKS : 2)
     } else {
       const bool has = idx < n_prim_gen;
       int note = 0;
-      if (has) alive = load_primary<R, true>(V, S, ctl->prim_begin + idx, book, t, note);
+      if (has) alive = load_primary<R, true>(V, S, ctl->plan.prim_begin + idx, book, t, note);
       count_primaries(row, has, t.type, note);
     }
-    const int K = ctl->K;
+    const int K = ctl->plan.K;
     for (int kk = 0; kk < K; ++kk) {
       if (!__any_sync(0xffffffffu, alive)) break;
       const bool was_alive = alive;
@@ -1697,10 +1706,9 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
   __shared__ View<R> sV;
   __shared__ WarpCnt s_wc[8];
   __shared__ unsigned s_kend[kNReqKey], s_kn[kNReqKey];
-  __shared__ int s_last;
   Ctl *ctl = S->ctl;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (ctl->done) return;
+  if (ctl->plan.done) return;
   if (tid == 0) {
     sV = S->view;  // tables stay in global memory: the final states read the alias bins only
     unsigned acc = 0;
@@ -1716,7 +1724,7 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
   __syncthreads();
   const View<R> &V = sV;
   const int out = parity ^ 1;
-  const bool book = ctl->book != 0;
+  const bool book = ctl->plan.book != 0;
   for (;;) {
     unsigned chunk = 0;
     if (lane == 0) chunk = atomicAdd(&ctl->claim_b, 1u);
@@ -1768,16 +1776,7 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
     if (v) atomicAdd(&ctl->counters[tid], v);
   }
   __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    const unsigned d = atomicAdd(&ctl->blocks_done_b, 1u);
-    s_last = (d == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (s_last && tid == 0) {
-    __threadfence();
-    plan_next(S, out);
-  }
+  if (tid == 0 && block_done(&ctl->blocks_done_b)) plan_next(S, out);
 }
 
 }  // namespace gv
@@ -2202,10 +2201,10 @@ template <typename R> DevState<R> make_state(Ctx *c) {
 // ends it earlier through plan_next).
 __global__ void loop_gate_kernel(Ctl *ctl, cudaGraphConditionalHandle h, unsigned long long max_iter) {
   const unsigned long long it = ++ctl->loop_iter;
-  int stop = ctl->done;
+  int stop = ctl->plan.done;
   if (!stop && it >= max_iter) {
     if (ctl->status == 0) ctl->status = GV_ERR_TIMEOUT;
-    ctl->done = 1;
+    ctl->plan.done = 1;
     stop = 1;
   }
   cudaGraphSetConditional(h, stop ? 0u : 1u);
@@ -2522,7 +2521,7 @@ int run_transport(Ctx *c, const gv_primary *p, long long n, long long first_even
       float ms = 0.f;
       CK(cudaEventElapsedTime(&ms, c->t0, c->t1));
       kernel_ms += ms;
-      if (c->h_ctl->done) break;
+      if (c->h_ctl->plan.done) break;
       between = std::min(between * 2, 64);
     }
   }
@@ -2920,7 +2919,7 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
       return GV_ERR_CUDA;
     if (batch == 0) continue;
     if (cudaEventSynchronize(seen[(batch - 1) & 1]) != cudaSuccess) return GV_ERR_CUDA;
-    if (*const_cast<volatile int *>(&c->h_ctl->done)) break;  // final once set, whichever batch it came with
+    if (*const_cast<volatile int *>(&c->h_ctl->plan.done)) break;  // final once set, whichever batch it came with
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) return GV_ERR_CUDA;
   for (int i = 0; i < 16; ++i) counters[i] = c->h_ctl->counters[i];
