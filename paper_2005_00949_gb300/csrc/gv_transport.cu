@@ -55,15 +55,22 @@ template <typename R> __device__ __forceinline__ void kahan_add(R &sum, R &comp,
   sum = t;
 }
 
+// A tally's addition, with nothing returned (atomicAdd waited for more than
+// that: 80 cycles of a step's 1500).
+__device__ __forceinline__ void red_add(double *p, double v) {
+  asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
+
+// row: the event's row of the sub-slab tally.
 // EXT: compiled with the cell histogram and the per-event counters; a
 // kernel without them serves contexts that have neither.
 template <typename R, bool EXT = true>
-__device__ __forceinline__ void deposit(const View<R> &V, const DevState<R> *S, unsigned ev, int sub, double px,
-                                        double py, R dE, Pending<R> *pd = nullptr) {
+__device__ __forceinline__ void deposit(const DevState<R> *S, double *row, unsigned ev, int sub, double px, double py,
+                                        R dE, Pending<R> *pd = nullptr) {
   if (!(dE != R(0)) || sub < 0) return;
-  GV_CHECK(&S->ctl->status, ev < S->n_events && sub < V.geo.nsub);
-  const unsigned long long key = static_cast<unsigned long long>(ev) * V.geo.nsub + sub;
+  GV_CHECK(&S->ctl->status, ev < S->n_events && sub < S->view.geo.nsub);
   if (pd) {
+    const unsigned long long key = static_cast<unsigned long long>(ev) * S->view.geo.nsub + sub;
     if (pd->key == key) {
       kahan_add(pd->sum, pd->comp, dE);
     } else {
@@ -74,10 +81,10 @@ __device__ __forceinline__ void deposit(const View<R> &V, const DevState<R> *S, 
       pd->comp = R(0);
     }
   } else {
-    atomicAdd(&S->edep[key], f2d(dE));
+    red_add(&row[sub], f2d(dE));
   }
   if (EXT && S->cell) {
-    const GeoConst &g = V.geo;
+    const GeoConst &g = S->view.geo;
     const int layer = sub / g.nsub_layer;
     // the offset from the wall in FP64, the cell index in FP32 (a cell
     // edge moves by ~1e-7 of the box width; no FP64 division)
@@ -85,7 +92,7 @@ __device__ __forceinline__ void deposit(const View<R> &V, const DevState<R> *S, 
     int iy = __float2int_rd(static_cast<float>(py + g.hy) * g.inv_pitch_y);
     ix = ix < 0 ? 0 : (ix >= g.nx ? g.nx - 1 : ix);
     iy = iy < 0 ? 0 : (iy >= g.ny ? g.ny - 1 : iy);
-    atomicAdd(&S->cell[(static_cast<size_t>(layer) * g.nx + ix) * g.ny + iy], f2d(dE));
+    red_add(&S->cell[(static_cast<size_t>(layer) * g.nx + ix) * g.ny + iy], f2d(dE));
   }
 }
 
@@ -161,12 +168,32 @@ template <typename R> struct Run {
   int note;
 };
 
+// The tables as the step kernels stage them (stage_tables), addressed from the
+// start of shared memory: through the view's pointers every load would be a
+// generic one, behind the load of the pointer, which the deposits' atomics
+// make the compiler repeat in every step.  What is the same for all tracks
+// (planes' count, half widths, cuts) the steps read from the state record in
+// constant memory, as operands.
+template <typename R> struct Staged {
+  const V4<R> *xs;
+  const double *zb;
+  const float *inv_node;
+  const SubRec<R> *rec;
+  __device__ __forceinline__ explicit Staged(const DevState<R> *S) {
+    extern __shared__ __align__(32) unsigned char smem[];
+    xs = reinterpret_cast<const V4<R> *>(smem);
+    zb = reinterpret_cast<const double *>(smem + S->xs_bytes);
+    inv_node = reinterpret_cast<const float *>(smem + S->xs_bytes + S->zb_bytes);
+    rec = reinterpret_cast<const SubRec<R> *>(smem + S->rec_off);
+  }
+};
+
 // A track left the box (or there is nothing left to stop it).
 template <typename R, bool EXT>
-__device__ __forceinline__ void escape(const View<R> &V, const DevState<R> *S, const Trk<R> &t, int plane, Run<R> &r) {
+__device__ __forceinline__ void escape(const DevState<R> *S, const Trk<R> &t, int plane, Run<R> &r) {
   atomicAdd(&S->escape[t.ev], f2d(t.E));
   if (t.type == 2) r.note |= kNoteEpEsc;
-  if ((t.flags & kFlagPrimary) && !(t.flags & kFlagInteracted) && plane == V.geo.nsub) r.note |= kNoteUnscat;
+  if ((t.flags & kFlagPrimary) && !(t.flags & kFlagInteracted) && plane == S->view.geo.nsub) r.note |= kNoteUnscat;
 }
 
 // Photons: PreStep to the end of a run of at most `budget` steps, every one
@@ -179,69 +206,81 @@ __device__ __forceinline__ void escape(const View<R> &V, const DevState<R> *S, c
 // no wall test while the run's lateral bound clears the plane (2000 x 10 GeV:
 // 5.39 -> 5.02 ms with the branch-free widening, the shared exponential of
 // loss_at and one-branch grid_pos).
+//
+// A run is one chain of dependent instructions, so the loop has one exit, and
+// the next sub-slab's record and cross sections are fetched before the exit is
+// decided (PHOTONTIME).
 template <typename R, bool EXT>
-__device__ __forceinline__ int photon_run(const View<R> &V, const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r) {
+__device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r) {
+  const Staged<R> V(S);
+  const GeoConst &geo = S->view.geo;
   int gi;
   R gf;
-  grid_pos(V, t.E, gi, gf);
-  const V4<R> *const tab = V.xs + gi;
   const R INF = r_inf<R>();
   const bool up = t.w > R(0), plane_ahead = t.w != R(0);
+  int sub = t.sub;
+  GV_CHECK(&S->ctl->status, sub >= 0 && sub < geo.nsub);
+  SubRec<R> rec = V.rec[sub];
+  R h = static_cast<R>(V.zb[up ? sub + 1 : sub] - t.z);
+  grid_pos_on(V.inv_node, t.E, gi, gf);
+  GV_CHECK(&S->ctl->status, gi >= 0 && gi <= kGridN - 2);
+  const V4<R> *const tab = V.xs + gi;
   const Divisor<R> by_w(t.w);
-  float lat = lateral_free(V, t.x, t.y);
-  int sub = t.sub, m = 0, end = kRunOn;
-  R nlam = t.nlam, s = R(0);
-  do {
-    const SubRec<R> rec = V.rec[sub];
-    const V4<R> *p = tab + rec.row;  // ComputeIntLen
-    GV_CHECK(&S->ctl->status, gi >= 0 && gi <= kGridN - 2 && sub >= 0 && sub < V.geo.nsub);
-    const V4<R> s4 = lerp4(p[0], p[1], gf);
-    r.sig0 = s4.x;
-    r.sig1 = s4.y;
-    r.sig2 = s4.z;
-    const R Sig = r.sig0 + r.sig1 + r.sig2;
+  float lat = lateral_free(geo, t.x, t.y);
+  const int last = geo.nsub - 1, dir = up ? 1 : -1;
+  V4<R> sig = lerp4(tab[rec.row], tab[rec.row + 1], gf);  // ComputeIntLen
+  R nlam = t.nlam, s;
+  int m = 0, pl;
+  bool finite, geom, out;
+  for (;;) {
+    const R Sig = sig.x + sig.y + sig.z;
     const R s_phys = Sig > R(0) ? q_div(nlam, Sig) : INF;
     // GeomQuery
-    R d = INF;
-    if (plane_ahead) {
-      const R h = m ? (up ? rec.thick : -rec.thick) : static_cast<R>(V.zb[up ? sub + 1 : sub] - t.z);
-      d = by_w.div(h);
-    }
-    int pl = -1;
-    walls(V, t.x, t.y, t.u, t.v, lat, d, pl);
+    R d = plane_ahead ? by_w.div(h) : INF;
+    const int next = sub + dir;
+    const SubRec<R> nrec = V.rec[min(max(next, 0), last)];
+    const V4<R> nsig = lerp4(tab[nrec.row], tab[nrec.row + 1], gf);
+    pl = -1;
+    walls(geo, t.x, t.y, t.u, t.v, lat, d, pl);
     const R s_geom = d < R(0) ? R(0) : d;
     s = INF < s_geom ? INF : s_geom;
     s = s_phys < s ? s_phys : s;
-    if (!(s < INF)) {
-      r.n_iter = 1;
-      end = kRunEnd;
-      escape<R, EXT>(V, S, t, -1, r);
-      break;
-    }
-    ++m;
+    finite = s < INF;
+    geom = s_geom == s;
+    out = pl < -1 || static_cast<unsigned>(next) > static_cast<unsigned>(last);
     t.x += f2d(s * t.u);
     t.y += f2d(s * t.v);
-    if (!(s_geom == s)) {  // physics (a photon has no other limit)
-      end = kRunPhys;
-      break;
-    }
-    ++r.n_geom;
-    if (Sig > R(0)) nlam = nlam - s * Sig;
     lat = lat_after(lat, s);
-    sub += up ? 1 : -1;
-    if (pl < -1 || static_cast<unsigned>(sub) >= static_cast<unsigned>(V.geo.nsub)) {
-      end = kRunEnd;
-      escape<R, EXT>(V, S, t, pl < -1 ? pl : (up ? V.geo.nsub : 0), r);
-      break;
+    ++m;
+    if (geom && Sig > R(0)) nlam = nlam - s * Sig;
+    if (!finite || !geom || out || !(nlam > R(0)) || m >= budget) break;
+    sub = next;
+    h = up ? nrec.thick : -nrec.thick;  // from the plane it enters through
+    sig = nsig;
+  }
+  r.sig0 = sig.x;
+  r.sig1 = sig.y;
+  r.sig2 = sig.z;
+  r.n_iter = static_cast<unsigned>(m);
+  if (!finite) --m;  // not a step: nothing stops the track
+  r.n_st = static_cast<unsigned>(m);
+  t.step += static_cast<unsigned>(m);
+  r.n_geom = static_cast<unsigned>(finite && !geom ? m - 1 : m);
+  int end = kRunOn;
+  if (!finite || (geom && out)) {
+    end = kRunEnd;
+    escape<R, EXT>(S, t, !finite || pl < -1 ? pl : (up ? geo.nsub : 0), r);
+  } else {
+    if (geom) sub += dir;
+    if (r.n_geom) t.z = V.zb[up ? sub : sub + 1];  // the plane it entered through
+    if (!geom) {  // physics (a photon has no other limit)
+      t.z += f2d(s * t.w);
+      nlam = R(0);
+      end = kRunPhys;
     }
-  } while (m < budget && nlam > R(0));
-  if (r.n_geom && end != kRunEnd) t.z = V.zb[up ? sub : sub + 1];  // the plane it entered through
-  if (end == kRunPhys) t.z += f2d(s * t.w);
+  }
   t.nlam = nlam;
   t.sub = sub;
-  t.step += static_cast<unsigned>(m);
-  r.n_st = static_cast<unsigned>(m);
-  r.n_iter = max(r.n_iter, r.n_st);
   return end;
 }
 
@@ -251,17 +290,25 @@ __device__ __forceinline__ int photon_run(const View<R> &V, const DevState<R> *S
 template <typename R, bool FIELD, bool OPTS, bool EXT>
 __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r,
                                            Pending<R> *pd) {
-  const R INF = r_inf<R>();
+  const Staged<R> T(S);
+  const GeoConst &geo = S->view.geo;
+  const R INF = r_inf<R>(), tcut = S->view.rc.tcut;
   const bool pos = t.type == 2;
-  float lat = lateral_free(V, t.x, t.y);
+  double *const edep = S->edep + static_cast<size_t>(t.ev) * geo.nsub;
+  float lat = lateral_free(geo, t.x, t.y);
   for (int m = 0; m < budget; ++m) {
     ++r.n_iter;
-    GV_CHECK(&S->ctl->status, t.sub >= 0 && t.sub < V.geo.nsub);
-    const V4<R> *const tab = V.xs + (V.rec[t.sub].row + (pos ? 2 * kGridN : kGridN));
+    GV_CHECK(&S->ctl->status, t.sub >= 0 && t.sub < geo.nsub);
+    // GeomQuery's plane difference first: it takes the FP64 pipe about as long
+    // as the lookups below take
+    const bool up = t.w > R(0);
+    int plane = up ? t.sub + 1 : t.sub;
+    const R dz = static_cast<R>(T.zb[plane] - t.z);
+    const V4<R> *const tab = T.xs + (T.rec[t.sub].row + (pos ? 2 * kGridN : kGridN));
     // ComputeIntLen; the pre-step energy's grid position serves the lookup and the loss
     int gi;
     R gf;
-    grid_pos(V, t.E, gi, gf);
+    grid_pos_on(T.inv_node, t.E, gi, gf);
     const V4<R> n0 = tab[gi], n1 = tab[gi + 1];
     const V4<R> s4 = lerp4(n0, n1, gf);
     r.sig0 = s4.x;
@@ -272,7 +319,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     // cross sections the track can reach; the interaction is accepted at the
     // post-step point
     R Smax = Sig;
-    if (OPTS && (V.cut.mask & GV_P_INTEGRAL)) {
+    if (OPTS && (S->view.cut.mask & GV_P_INTEGRAL)) {
       const R *mx = V.smax + (V.smat[t.sub] * 2 + t.type - 1) * kGridN;
       Smax = mx[gi] + gf * (mx[gi + 1] - mx[gi]);
     }
@@ -281,18 +328,23 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     const R Rr = range_of(s4, t.type);
     const R a = static_cast<R>(kAlphaR) * Rr, b = Rr < static_cast<R>(kRhoF) ? Rr : static_cast<R>(kRhoF);
     R s_cont = a > b ? a : b;
-    if (FIELD && V.rc.field_k != R(0)) {  // the field's step limit acts like the continuous one
+    if (FIELD && S->view.rc.field_k != R(0)) {  // the field's step limit acts like the continuous one
       const R sf = field_limit(V, t.type, t.E, t.u, t.v, t.w);
       s_cont = sf < s_cont ? sf : s_cont;
     }
     // GeomQuery
-    int next, plane;
-    const R s_geom = distance(V, t.x, t.y, t.z, t.u, t.v, t.w, t.sub, lat, next, plane);
+    int next = up ? t.sub + 1 : t.sub - 1;
+    R s_geom = INF;
+    if (t.w != R(0)) s_geom = q_div(dz, t.w);
+    else plane = -1;
+    walls(geo, t.x, t.y, t.u, t.v, lat, s_geom, plane);
+    if (plane < -1 || next >= geo.nsub) next = -1;
+    if (s_geom < R(0)) s_geom = R(0);
     R s = s_cont < s_geom ? s_cont : s_geom;
     s = s_phys < s ? s_phys : s;
     const int lim = (s_geom == s) ? 0 : (s_phys == s ? 1 : 2);
     if (!(s < INF)) {
-      escape<R, EXT>(V, S, t, -1, r);
+      escape<R, EXT>(S, t, -1, r);
       return kRunEnd;
     }
     // Propagation: FP64 positions, advanced by displacements s d formed in R
@@ -300,7 +352,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     // integer ALU, leaving the FP64 pipe one addition per coordinate; in FP64
     // mode this is one fused multiply-add)
     double mx = 0.0, my = 0.0;  // step midpoint: only cell scoring reads it
-    if (FIELD && V.rc.field_k != R(0)) {  // the helix of the pre-step momentum
+    if (FIELD && S->view.rc.field_k != R(0)) {  // the helix of the pre-step momentum
       const R d0[3] = {t.u, t.v, t.w};
       R dp[3], nd[3];
       if (EXT && S->cell) {
@@ -313,9 +365,9 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       t.y += f2d(dp[1]);
       t.z += f2d(dp[2]);
       if (lim == 0) {  // the crossed plane, chosen with the pre-step direction
-        if (plane >= 0) t.z = V.zb[plane];
-        else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
-        else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
+        if (plane >= 0) t.z = T.zb[plane];
+        else if (plane == -2) t.x = t.u > R(0) ? geo.wx[1] : geo.wx[0];
+        else if (plane == -3) t.y = t.v > R(0) ? geo.wy[1] : geo.wy[0];
       }
       t.u = nd[0];
       t.v = nd[1];
@@ -329,9 +381,9 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       t.y += f2d(s * t.v);
       t.z += f2d(s * t.w);
       if (lim == 0) {
-        if (plane >= 0) t.z = V.zb[plane];
-        else if (plane == -2) t.x = V.geo.wx[t.u > R(0) ? 1 : 0];
-        else if (plane == -3) t.y = V.geo.wy[t.v > R(0) ? 1 : 0];
+        if (plane >= 0) t.z = T.zb[plane];
+        else if (plane == -2) t.x = t.u > R(0) ? geo.wx[1] : geo.wx[0];
+        else if (plane == -3) t.y = t.v > R(0) ? geo.wy[1] : geo.wy[0];
       }
     }
     if (Smax > R(0)) t.nlam = (lim == 1) ? R(0) : t.nlam - s * Smax;
@@ -345,15 +397,15 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     const R Li = pos ? n0.w : n0.z;
     const Loss<R> loss = loss_at(tab, t.type, t.E, gi, gf, Li, (pos ? n1.w : n1.z) - Li, s, Rr);
     const R Ep = loss_energy(loss);
-    deposit<R, EXT>(V, S, t.ev, pre_sub, mx, my, t.E - Ep, pd);
+    deposit<R, EXT>(S, edep, t.ev, pre_sub, mx, my, t.E - Ep, pd);
     t.E = Ep;
     lat = lat_after(lat, s);
-    if (t.E < V.rc.tcut) {
-      deposit<R, EXT>(V, S, t.ev, pre_sub, t.x, t.y, t.E, pd);
+    if (t.E < tcut) {
+      deposit<R, EXT>(S, edep, t.ev, pre_sub, t.x, t.y, t.E, pd);
       return t.type == 2 ? kRunRest : kRunEnd;
     }
     // multiple scattering of a track that stays in the box (counter block 2)
-    if (OPTS && (V.cut.mask & GV_P_MSC) && !(lim == 0 && next < 0)) {
+    if (OPTS && (S->view.cut.mask & GV_P_MSC) && !(lim == 0 && next < 0)) {
       const uint4 r2 = track_draw(S, t.id, t.ev, k, 2u);
       const R um[4] = {u24<R>(r2.x), u24<R>(r2.y), u24<R>(r2.z), u24<R>(r2.w)};
       R dm[3] = {t.u, t.v, t.w};
@@ -361,11 +413,11 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       t.u = dm[0];
       t.v = dm[1];
       t.w = dm[2];
-      lat = lateral_free(V, t.x, t.y);  // the lateral offset is not part of the step
+      lat = lateral_free(geo, t.x, t.y);  // the lateral offset is not part of the step
     }
     if (lim == 0) {
       if (next < 0) {
-        escape<R, EXT>(V, S, t, plane, r);
+        escape<R, EXT>(S, t, plane, r);
         return kRunEnd;
       }
       t.sub = next;
@@ -401,11 +453,11 @@ __device__ __forceinline__ int run_round(const View<R> &V, const DevState<R> *S,
   if (t.E < V.rc.tcut) {  // PreStep: tracking cut
     r.n_iter = 1;
     kk = t.step;
-    deposit<R, EXT>(V, S, t.ev, t.sub, t.x, t.y, t.E, pd);
+    deposit<R, EXT>(S, S->edep + static_cast<size_t>(t.ev) * S->view.geo.nsub, t.ev, t.sub, t.x, t.y, t.E, pd);
     end = t.type == 2 ? kRunRest : kRunEnd;
   } else {
     if (t.nlam <= R(0)) t.nlam = -m_log(u24<R>(track_draw(S, t.id, t.ev, t.step, 0u).x));
-    end = t.type == 0 ? photon_run<R, EXT>(V, S, t, budget_g, r)
+    end = t.type == 0 ? photon_run<R, EXT>(S, t, budget_g, r)
                       : charged_run<R, FIELD, OPTS, EXT>(V, S, t, budget, r, pd);
     kk = t.step - 1u;
   }
@@ -475,7 +527,7 @@ __device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *
                       S->seed_hi};
     r = interact<R, OPTS, ALT>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na);
     if (r < 0) return -1;
-    deposit<R, EXT>(V, S, ev, sub, x, y, local, pd);
+    deposit<R, EXT>(S, S->edep + static_cast<size_t>(ev) * S->view.geo.nsub, ev, sub, x, y, local, pd);
   }
   if (EXT && S->evcnt) {
     unsigned long long *row = &S->evcnt[static_cast<size_t>(ev) * GV_NCOUNT];
