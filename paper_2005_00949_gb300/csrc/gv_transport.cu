@@ -523,13 +523,16 @@ __device__ __forceinline__ int run_round(const View<R> &V, const DevState<R> *S,
 // PostStepActions of the request `key`: the final state and its local
 // deposit.  Returns 1 if the particle survives, 0 if it ended, -1 if the
 // process was kinematically closed at the post-step energy (nothing
-// changes).  np, na: pairs and annihilations made.
+// changes).  np, na: pairs and annihilations made.  ids: the words that name
+// its first two secondaries (push_kids), drawn with its own numbers: the two
+// chains of Philox rounds run side by side.
 template <typename R, bool OPTS = true, bool EXT = true, bool ALT = false>
 __device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *S, int key, R &E, R d[3], R u2, R u3,
                                            Kids<R> &kids, unsigned ev, int sub, double x, double y,
                                            unsigned long long id, uint32_t kk, int &np, int &na,
-                                           Pending<R> *pd = nullptr) {
+                                           uint4 &ids, Pending<R> *pd = nullptr) {
   const uint4 r1 = track_draw(S, id, ev, kk, 1u);
+  ids = track_draw(S, id, ev, kk, kTagId);
   const R u[8] = {R(0), R(0), u2, u3, u24<R>(r1.x), u24<R>(r1.y), u24<R>(r1.z), u24<R>(r1.w)};
   int r = 0;
   if (key == kKeyRest) {
@@ -763,14 +766,14 @@ template <typename R> struct LocalStack {
 // 32 lanes of a converged warp (lanes without secondaries pass kids.n == 0).
 template <typename R, bool EXT = true>
 __device__ __forceinline__ void push_kids(const DevState<R> *S, int out, const Parent &t, const Kids<R> &kids,
-                                          uint32_t kk, unsigned long long *row, const LocalStack<R> *ls = nullptr) {
+                                          uint32_t kk, const uint4 &ids, unsigned long long *row,
+                                          const LocalStack<R> *ls = nullptr) {
   const unsigned b0 = __ballot_sync(0xffffffffu, kids.n > 0);
   if (!b0) return;
   const int lane = threadIdx.x & 31;
   uint32_t w[6] = {0, 0, 0, 0, 0, 0};
   if (kids.n > 0) {
-    const uint4 a = track_draw(S, t.id, t.ev, kk, kTagId);
-    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+    w[0] = ids.x; w[1] = ids.y; w[2] = ids.z; w[3] = ids.w;
     if (kids.n > 2) {
       const uint4 b = track_draw(S, t.id, t.ev, kk, kTagId + 1u);
       w[4] = b.x; w[5] = b.y;
@@ -1491,11 +1494,12 @@ __global__ void GV_STEP_BOUNDS
       if (!SORT) {  // final state in place (warp-divergent across processes)
         Kids<R> kids;
         kids.n = 0;
+        uint4 ids = make_uint4(0u, 0u, 0u, 0u);
         int np = 0, na = 0, change = own_end ? -1 : 0;
         if (key >= 0) {
           R d[3] = {t.u, t.v, t.w};
           const int r = final_state<R, OPTS, EXT, ALT>(V, S, key, t.E, d, u2, u3, kids, t.ev, t.sub, t.x, t.y, t.id, kstep, np,
-                                                  na, pd);
+                                                  na, ids, pd);
           if (r >= 0) {
             t.u = d[0]; t.v = d[1]; t.w = d[2];
             t.flags |= kFlagInteracted;
@@ -1506,7 +1510,7 @@ __global__ void GV_STEP_BOUNDS
         wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
         wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
         if (book && book_live(S, t.ev, change) == 1u) event_closed(S, t.ev);
-        push_kids<R, EXT>(S, out, Parent{t.x, t.y, t.z, t.id, t.ev, t.sub}, kids, kstep, row);
+        push_kids<R, EXT>(S, out, Parent{t.x, t.y, t.z, t.id, t.ev, t.sub}, kids, kstep, ids, row);
         if (MERGE) warp_flush(S, pend);
         continue;
       }
@@ -1570,6 +1574,7 @@ __global__ void GV_STEP_BOUNDS
         kb.n = 0;
         Parent par;
         uint32_t pk = 0;
+        uint4 ids = make_uint4(0u, 0u, 0u, 0u);
         int np = 0, na = 0;
         if (static_cast<unsigned>(tid) < nreq) {
           const double2 a = req.xy(tid), c = req.zi(tid);
@@ -1583,7 +1588,7 @@ __global__ void GV_STEP_BOUNDS
           R d[3] = {dE.x, dE.y, dE.z};
           R e = dE.w;
           const int r = final_state<R, OPTS, EXT, ALT>(V, S, static_cast<int>(g.w), e, d, req.u2(tid), req.u3(tid), kb, par.ev,
-                                                  par.sub, par.x, par.y, par.id, pk, np, na);
+                                                  par.sub, par.x, par.y, par.id, pk, np, na, ids);
           req.dir(tid) = V4<R>{d[0], d[1], d[2], e};
           req.ret(tid) = r;
           if (book) {
@@ -1593,7 +1598,7 @@ __global__ void GV_STEP_BOUNDS
         }
         wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
         wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
-        push_kids<R, EXT>(S, out, par, kb, pk, row, use_local ? &lstk : nullptr);
+        push_kids<R, EXT>(S, out, par, kb, pk, ids, row, use_local ? &lstk : nullptr);
       }
       __syncthreads();
       if (key >= 0 && key != kKeyRest) {
@@ -1806,6 +1811,7 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
     kids.n = 0;
     Parent par = {0.0, 0.0, 0.0, 0ull, 0u, 0};
     uint32_t kk = 0;
+    uint4 ids = make_uint4(0u, 0u, 0u, 0u);
     int np = 0, na = 0;
     unsigned was = 0u;
     bool alive = false;
@@ -1822,7 +1828,7 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
       kk = q.kk;
       t.step = kk + 1;
       t.nlam = R(-1);
-      const int r = final_state<R>(V, S, k, e, d, q.u2, q.u3, kids, t.ev, t.sub, t.x, t.y, q.id, q.kk, np, na);
+      const int r = final_state<R>(V, S, k, e, d, q.u2, q.u3, kids, t.ev, t.sub, t.x, t.y, q.id, q.kk, np, na, ids);
       t.E = e;
       t.u = d[0]; t.v = d[1]; t.w = d[2];
       if (r >= 0) t.flags |= kFlagInteracted;
@@ -1832,7 +1838,7 @@ __global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__rest
     }
     wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
     wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
-    push_kids<R>(S, out, par, kids, kk, row);
+    push_kids<R>(S, out, par, kids, kk, ids, row);
     push_track(S, out, t, alive);
     if (was == 1u) event_closed(S, t.ev);
   }
