@@ -858,6 +858,62 @@ __device__ __forceinline__ void push_kids(const DevState<R> *S, int out, const P
   }
 }
 
+// The end of a claim: the secondaries of the final states the warp ran (t's
+// are its own) and its lanes' survivors, appended with one reservation: a trip
+// to L2 less per claim, and the block does not wait at the results barrier for
+// the warps that append secondaries (2000 x 10 GeV: 4.16 -> 3.99 ms).  All 32
+// lanes of a converged warp.
+template <typename R, bool EXT = true>
+__device__ __forceinline__ void push_all(const DevState<R> *S, int out, const Parent &p, const Kids<R> &kids,
+                                         const uint4 &ids, uint32_t kk, const Trk<R> &t, bool alive,
+                                         unsigned long long *row) {
+  uint32_t w[6] = {ids.x, ids.y, ids.z, ids.w, 0u, 0u};
+  if (kids.n > 2) {
+    const uint4 b = track_draw(S, p.id, p.ev, kk, kTagId + 1u);
+    w[4] = b.x; w[5] = b.y;
+  }
+  WarpAppend ap;
+  unsigned rank[3] = {0, 0, 0};
+  bool some[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    some[j] = __any_sync(0xffffffffu, j < kids.n);
+    if (some[j]) rank[j] = ap.add(j < kids.n, kids.type[j]);
+  }
+  if (some[0]) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) wcnt_add(row, GV_C_TRK_G + q, ap.n[q]);
+    if (EXT && S->evcnt) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (j < kids.n) atomicAdd(&S->evcnt[static_cast<size_t>(p.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
+    }
+  }
+  const unsigned srank = ap.add(alive, t.type);
+  const unsigned base = ap.reserve(S->ctl->cnt[out]);
+  const unsigned slot = WarpAppend::slot(base, alive ? t.type : 0, srank);
+  bool full = false;
+  if (alive) {
+    if (slot < S->capacity)
+      store_track<R>(S, out, t.type, slot, t.x, t.y, t.z, t.u, t.v, t.w, t.E, t.nlam, t.id, t.ev, t.step,
+                     t.sub | (t.flags << 16));
+    else full = true;
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (!some[j]) continue;
+    const bool has = j < kids.n;
+    const unsigned ks = WarpAppend::slot(base, has ? kids.type[j] : 0, rank[j]);
+    if (!has) continue;
+    if (ks < S->capacity)
+      store_track<R>(S, out, kids.type[j], ks, p.x, p.y, p.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j], R(-1),
+                     static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
+                     p.ev, 0u, p.sub);
+    else full = true;
+  }
+  if (full) set_status(S->ctl, GV_ERR_STACK_FULL);
+}
+
 // Survivors: one record per lane (has: whether it has one).  All 32 lanes of
 // a converged warp.
 template <typename R>
@@ -1463,7 +1519,8 @@ __global__ void GV_STEP_BOUNDS
     }
     const int K = s_plan.K;
     unsigned ended_own = 0u, ended_req = 0u;  // evlive before this lane's last bookings of an end (1: the event closed)
-    unsigned ev_req = 0u;
+    unsigned ev_req = 0u, next_chunk = 0u;
+    bool claimed = false;
     for (int kk = 0; kk < K; ++kk) {
       // (with the basketizer the block leaves the loop together, after the
       // count barrier below shows that no lane was alive)
@@ -1569,12 +1626,12 @@ __global__ void GV_STEP_BOUNDS
         req.u3(slot) = u3;
       }
       __syncthreads();
+      Kids<R> kb;
+      kb.n = 0;
+      Parent par;
+      uint32_t pk = 0;
+      uint4 ids = make_uint4(0u, 0u, 0u, 0u);
       {
-        Kids<R> kb;
-        kb.n = 0;
-        Parent par;
-        uint32_t pk = 0;
-        uint4 ids = make_uint4(0u, 0u, 0u, 0u);
         int np = 0, na = 0;
         if (static_cast<unsigned>(tid) < nreq) {
           const double2 a = req.xy(tid), c = req.zi(tid);
@@ -1598,7 +1655,9 @@ __global__ void GV_STEP_BOUNDS
         }
         wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
         wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
-        push_kids<R, EXT>(S, out, par, kb, pk, ids, row, use_local ? &lstk : nullptr);
+        // with more rounds to come the secondaries go out (or on the stack) now;
+        // the last round's wait for the survivors
+        if (kk + 1 < K) push_kids<R, EXT>(S, out, par, kb, pk, ids, row, use_local ? &lstk : nullptr);
       }
       __syncthreads();
       if (key >= 0 && key != kKeyRest) {
@@ -1610,23 +1669,21 @@ __global__ void GV_STEP_BOUNDS
           alive = r != 0;
         }
       }
-      if (book) {  // the last round's are read after the survivors are out
-        if (own_end) ended_own = book_live(S, t.ev, -1);
-        if (kk + 1 < K) {
-          if (ended_own == 1u) event_closed(S, t.ev);
-          if (ended_req == 1u) event_closed(S, ev_req);
-          ended_own = ended_req = 0u;
-        }
+      if (book && own_end) ended_own = book_live(S, t.ev, -1);
+      if (kk + 1 == K) {
+        // the next claim's atomic is in flight while the claim's tracks go out
+        if (tid == 0) next_chunk = gridDim.x + atomicAdd(&ctl->claim.n, 1u);
+        claimed = true;
+        push_all<R, EXT>(S, out, par, kb, ids, pk, t, alive, row);
       }
+      // (the event counts' atomics were in flight while the tracks went out)
+      if (ended_own == 1u) event_closed(S, t.ev);
+      if (ended_req == 1u) event_closed(S, ev_req);
+      ended_own = ended_req = 0u;
     }
-    // the next claim's atomic and the event count's are in flight while the
-    // survivors are written
-    unsigned next_chunk = 0u;
-    if (block_claims && tid == 0) next_chunk = gridDim.x + atomicAdd(&ctl->claim.n, 1u);
+    if (block_claims && !claimed && tid == 0) next_chunk = gridDim.x + atomicAdd(&ctl->claim.n, 1u);
     if (MERGE) warp_flush(S, pend);  // nothing stays pending past a claim
-    push_track(S, out, t, alive);
-    if (ended_own == 1u) event_closed(S, t.ev);
-    if (ended_req == 1u) event_closed(S, ev_req);
+    if (!SORT) push_track(S, out, t, alive);
     if (use_local) {  // what is left on the block's stack goes to the next generation
       __syncthreads();
       const unsigned ng = s_stack.used & 0xffffu, nq = s_stack.used >> 16;
