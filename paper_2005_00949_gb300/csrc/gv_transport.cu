@@ -297,7 +297,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
   const Staged<R> T(S);
   const GeoConst &geo = S->view.geo;
   const R INF = r_inf<R>(), tcut = S->view.rc.tcut;
-  const bool pos = t.type == 2;
+  const bool pos = t.type == 2, msc = OPTS && (S->view.cut.mask & GV_P_MSC);
   double *const edep = S->edep + static_cast<size_t>(t.ev) * geo.nsub;
   GV_CHECK(&S->ctl->status, t.sub >= 0 && t.sub < geo.nsub);
   float lat = lateral_free(geo, t.x, t.y);
@@ -316,6 +316,9 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     ++r.n_iter;
     const int next = wall < -1 ? -1 : (t.w > R(0) ? (t.sub + 1 < geo.nsub ? t.sub + 1 : -1) : t.sub - 1);
     const V4<R> *const tab = T.xs + row;
+    // the scattering's numbers of this step (counter block 2), early
+    uint4 r2 = make_uint4(0u, 0u, 0u, 0u);
+    if (msc) r2 = track_draw(S, t.id, t.ev, t.step, 2u);
     // ComputeIntLen; the pre-step energy's grid position serves the lookup and the loss
     int gi;
     R gf;
@@ -339,8 +342,10 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     const R Rr = range_of(s4, t.type);
     const R a = static_cast<R>(kAlphaR) * Rr, b = Rr < static_cast<R>(kRhoF) ? Rr : static_cast<R>(kRhoF);
     R s_cont = a > b ? a : b;
+    R curv = R(0);
     if (FIELD && S->view.rc.field_k != R(0)) {  // the field's step limit acts like the continuous one
-      const R sf = field_limit(V, t.type, t.E, t.u, t.v, t.w);
+      curv = field_curv(S->view.rc.field_k, t.type, t.E);
+      const R sf = field_limit(geo.field_axis, curv, t.u, t.v, t.w);
       s_cont = sf < s_cont ? sf : s_cont;
     }
     R s = s_cont < s_geom ? s_cont : s_geom;
@@ -361,11 +366,11 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       const R d0[3] = {t.u, t.v, t.w};
       R dp[3], nd[3];
       if (EXT && S->cell) {
-        helix(V, t.type, t.E, R(0.5) * s, d0, dp, nd);
+        helix(geo.field_axis, curv, R(0.5) * s, d0, dp, nd);
         mx = t.x + f2d(dp[0]);
         my = t.y + f2d(dp[1]);
       }
-      helix(V, t.type, t.E, s, d0, dp, nd);
+      helix(geo.field_axis, curv, s, d0, dp, nd);
       t.x += f2d(dp[0]);
       t.y += f2d(dp[1]);
       t.z += f2d(dp[2]);
@@ -386,12 +391,11 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     if (lim == 0 && wall == -1) t.z = T.zb[crossed];
     const int pre_sub = t.sub, sub = lim == 0 && next >= 0 ? next : t.sub;
     plane = t.w > R(0) ? sub + 1 : sub;
-    dz = static_cast<R>(T.zb[plane] - t.z);
+    if (!msc) dz = static_cast<R>(T.zb[plane] - t.z);
     row = T.rec[sub].row + (pos ? 2 * kGridN : kGridN);
     lat = lat_after(lat, s);
     if (Smax > R(0)) t.nlam = (lim == 1) ? R(0) : t.nlam - s * Smax;
-    const uint32_t k = t.step;
-    t.step = k + 1;
+    ++t.step;
     ++r.n_st;
     r.n_geom += lim == 0 ? 1u : 0u;
     const R E_pre = t.E;
@@ -408,15 +412,14 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       break;
     }
     // multiple scattering of a track that stays in the box (counter block 2)
-    if (OPTS && (S->view.cut.mask & GV_P_MSC) && !(lim == 0 && next < 0)) {
-      const uint4 r2 = track_draw(S, t.id, t.ev, k, 2u);
+    if (msc && !(lim == 0 && next < 0)) {
       const R um[4] = {u24<R>(r2.x), u24<R>(r2.y), u24<R>(r2.z), u24<R>(r2.w)};
       R dm[3] = {t.u, t.v, t.w};
-      msc_step(V, pre_sub, E_pre, t.E, s, dm, t.x, t.y, t.z, um);
+      msc_step(geo, T.zb[pre_sub], T.zb[pre_sub + 1], S->view.rc.inv_X0[V.smat[pre_sub]], E_pre, t.E, s, dm, t.x, t.y,
+               t.z, um, lat);
       t.u = dm[0];
       t.v = dm[1];
       t.w = dm[2];
-      lat = lateral_free(geo, t.x, t.y);  // the lateral offset is not part of the step
       plane = t.w > R(0) ? sub + 1 : sub;
       dz = static_cast<R>(T.zb[plane] - t.z);
       by_w = Divisor<R>(t.w);

@@ -124,7 +124,9 @@ __global__ void k_msc(View<R> V, const int *sub, const double *Ea, const double 
   const R uu[4] = {static_cast<R>(u[4 * i]), static_cast<R>(u[4 * i + 1]), static_cast<R>(u[4 * i + 2]),
                    static_cast<R>(u[4 * i + 3])};
   double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
-  msc_step(V, sub[i], static_cast<R>(Ea[i]), static_cast<R>(Eb[i]), static_cast<R>(sv[i]), d, x, y, z, uu);
+  float lat = lateral_free(V.geo, x, y);
+  msc_step(V.geo, V.zb[sub[i]], V.zb[sub[i] + 1], V.rc.inv_X0[V.smat[sub[i]]], static_cast<R>(Ea[i]),
+           static_cast<R>(Eb[i]), static_cast<R>(sv[i]), d, x, y, z, uu, lat);
   od[3 * i] = d[0];
   od[3 * i + 1] = d[1];
   od[3 * i + 2] = d[2];
@@ -141,12 +143,13 @@ __global__ void k_field(View<R> V, int type, const double *E, const double *sv, 
   const R d[3] = {static_cast<R>(dir[3 * i]), static_cast<R>(dir[3 * i + 1]), static_cast<R>(dir[3 * i + 2])};
   R dp[3], nd[3];
   const R e = static_cast<R>(E[i]);
-  helix(V, type, e, static_cast<R>(sv[i]), d, dp, nd);
+  const R k = field_curv(V.rc.field_k, type, e);
+  helix(V.geo.field_axis, k, static_cast<R>(sv[i]), d, dp, nd);
   for (int j = 0; j < 3; ++j) {
     out[7 * i + j] = dp[j];
     out[7 * i + 3 + j] = nd[j];
   }
-  out[7 * i + 6] = field_limit(V, type, e, d[0], d[1], d[2]);
+  out[7 * i + 6] = V.rc.field_k == R(0) ? r_inf<R>() : field_limit(V.geo.field_axis, k, d[0], d[1], d[2]);
 }
 
 template <typename R>

@@ -78,3 +78,28 @@ def test_event_bookkeeping_follows_the_in_flight_cap(cap):
         assert np.array_equal(out[-1]["counts"][:, :11], out[0]["counts"][:, :11]), kw
     if cap:  # three events in flight take many more generations than all at once
         assert out[1]["counters"]["generations"] > 2 * out[0]["counters"]["generations"]
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("tesla", [1e-12, 1e-34, 1e-37, 1e-40])
+def test_field_too_weak_to_turn_a_step(precision, tesla):
+    """Turns down to the subnormal numbers and zero: the step is the straight
+    one (its own rounding, three products and two sums: 5 half-ulps; and the
+    turn itself, 0.29 / cm of a 10 MeV track in 1 T, where it is a number)."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    wl = W.with_field(W.pbps_electrons(1), tesla, 1)
+    ctx = gv.Context(wl, gv.gv_default_config(precision=precision, stack_capacity=1 << 12))
+    n = 64
+    s = np.repeat(10.0 ** np.arange(-14.0, 2.0), 4)
+    d = np.tile([[0.6, 0.0, 0.8], [0.0, 1.0, 0.0], [0.48, 0.6, -0.64], [0.0, 0.0, 1.0]], (n // 4, 1))
+    dev = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")
+    out = torch.zeros((n, 7), dtype=torch.float64, device="cuda")
+    ctx.gv_unit_field(1, dev(np.full(n, 10.0)), dev(s), dev(d), out)
+    g = out.cpu().numpy()
+    ctx.close()
+    eps = 2.0 ** (-22 if precision == 0 else -51)
+    assert (np.abs(g[:, :3] - s[:, None] * d) <= eps * s[:, None] + tesla * s[:, None] ** 2).all()
+    assert (np.abs(g[:, 3:6] - d) <= eps + tesla * s[:, None]).all()
