@@ -178,8 +178,10 @@ __global__ void k_sample(View<R> V, int model, int method, const double *E, long
 // it (ncu: L1 75 %, issue 61 %, DRAM 23 %); a random 16-byte read of shared
 // memory passes a warp in about 12 cycles.  4M pair samples: 44 -> 37 us.
 constexpr int kTabThreads = 1024;
-// below this many samples a block's copy of the rows costs more than it saves
-constexpr long long kTabMin = 1 << 18;
+// Below this many samples a block's copy of the rows costs more than it saves:
+// 2^18 samples take 8.1 us this way and 7.6 us through L1, 2^19 10.1 and
+// 9.9, 2^20 13.4 and 14.6, 2^22 37 and 45 (the mean of three models' tables).
+constexpr long long kTabMin = 1 << 20;
 
 __global__ void __launch_bounds__(kTabThreads, 2)
     k_sample_tab(const __grid_constant__ View<float> V, int model, const double *E, long long n, uint32_t k0, uint32_t k1,

@@ -70,12 +70,12 @@ def test_tallies_in_place_or_copied(gvmod, where):
 
 @pytest.mark.parametrize("model", range(6))
 def test_sampler_kernels_agree_at_their_border(gvmod, model):
-    """From 2^18 samples on the sampling tables are read from shared memory:
+    """From 2^20 samples on the sampling tables are read from shared memory:
     the same tables and arithmetic in another kernel, so equal up to the
     rounding of separately compiled FP32 code (a few ulp), except where that
     decides a table bin (bounded at 1e-4 of the samples)."""
     import torch
-    border = 1 << 18
+    border = 1 << 20
     wl = W.pbps_electrons(1)
     ctx = gvmod.Context(wl, gvmod.gv_default_config(stack_capacity=1 << 12))
     n = border + 77
