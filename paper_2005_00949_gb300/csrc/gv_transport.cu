@@ -55,8 +55,8 @@ template <typename R> __device__ __forceinline__ void kahan_add(R &sum, R &comp,
   sum = t;
 }
 
-// A tally's addition, with nothing returned (atomicAdd waited for more than
-// that: 80 cycles of a step's 1500).
+// A tally's addition, with nothing returned (an atomicAdd here cost a charged
+// step 80 cycles, of 1500 at the time and 950 now).
 __device__ __forceinline__ void red_add(double *p, double v) {
   asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
@@ -1231,8 +1231,8 @@ template <typename R> __global__ void init_kernel(const DevState<R> *S) { start_
 // turns those into prefix sums (pcost[i] = sum of prim_cost over primaries 0
 // .. i-1, for the automatic events-in-flight cap) and starts the control
 // block.  One block scanning all primaries after a copy and up to seven
-// memsets took 300 us for 1e5 photons, half of a 600 us transport (now 310
-// us); one shower takes 10 us less, of 870.
+// memsets took 300 us for 1e5 photons, half of a 600 us transport (300 us
+// now, of which the step kernels take 230); one shower takes 10 us less.
 constexpr int kPrepThreads = 256;
 constexpr int kScanBlocks = 304;  // scan blocks at most: two per SM
 struct Clear {
@@ -1371,9 +1371,10 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 // ------------------------------------------------------------------ the kernel
 // Register budget: GV_MIN_BLOCKS resident 256-thread blocks per SM in FP32
 // (measured: with the along-step loop 2 blocks at up to 128 registers beat
-// 3 blocks at 80 registers, which spill ~700 bytes).  FP64 runs one block
-// per SM without a register cap (222 registers, no spills; 4 % faster than
-// two blocks at 128 registers, which spilled).
+// 3 blocks at 80 registers, which spill 400 bytes: 14.9 ms against 13.3 on
+// the mixed-type batch).  FP64 runs one block per SM without a register cap
+// (192 to 240 registers, no spills; 4 % faster than two blocks at 128
+// registers, which spilled).
 // GV_MAX_BLOCK is the largest block the kernels are compiled for.
 #ifndef GV_MIN_BLOCKS
 #define GV_MIN_BLOCKS 2
@@ -1388,18 +1389,23 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 #define GV_STEP_BOUNDS __launch_bounds__(GV_MAX_BLOCK, sizeof(R) == 4 ? GV_MIN_BLOCKS : 1)
 #endif
 
-//
-// What bounds it: the instruction issue and the latency chains of a round at
-// the two blocks per SM that its registers allow (ncu: issue active 30 %, no
-// memory or FP64 pipe above 25 %).  So the work is cut where few lanes did it:
-// random numbers once per round instead of once per step (run_round), one
-// place that makes secondaries (a stopped positron is a request like any
-// other), counters booked by ballots into words of the warp (a 64-bit
-// shared-memory atomic is a loop), 16-byte track parts, one reservation
-// atomic for the three queues.  2000 x 10 GeV e- in Pb/polystyrene: 7.63 ->
-// 5.39 ms a transport; 1000 x 1 GeV: 1.41 -> 1.13 ms; 300 x 10 GeV in FP64:
-// 13.4 -> 10.8 ms (its arithmetic sits on the FP64 pipe); 2000 x 100 GeV in
-// W/Si with cells: 95.6 -> 65.5 ms.
+// What bounds it: the dependent chains of a round at the two blocks per SM
+// that its registers allow, and at a block's barriers its slowest warp.  At
+// the shower maximum (ncu, 500 x 10 GeV) a scheduler issues in 33 % of its
+// cycles; per issue 2.4 warps wait for L2, 2.1 for a fixed-latency result,
+// 2.0 at a barrier, 1.9 for shared memory and 0.8 for instructions (the code
+// is 110 KB); ALU 25 %, FP64 pipe 14 %, FMA 12 %, L2 6 %, DRAM 4 % of their
+// peaks.  FP64 kernels sit on the FP64 pipe (69 % at the maximum).  So the
+// chains are short and work is done where many lanes do it: random numbers
+// once per round instead of once per step (run_round), one place that makes
+// secondaries (a stopped positron is a request like any other), counters
+// booked by ballots into words of the warp (a 64-bit shared-memory atomic is
+// a loop), 16-byte track parts, one reservation atomic for the three queues,
+// a warp to a model (the sort below), a generation's plan in one read.  What a
+// caller waits for, before these and with them: 2000 x 10 GeV e- in
+// Pb/polystyrene 7.75 -> 3.98 ms, 1000 x 1 GeV 1.37 -> 0.72 ms, one 10 GeV
+// shower 1.13 -> 0.59 ms, 300 x 10 GeV in FP64 13.0 -> 8.5 ms, 2000 x 100 GeV
+// in W/Si with cells 94.8 -> 52.2 ms.
 template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT, bool ALT = !SORT>
 __global__ void GV_STEP_BOUNDS
     step_kernel(int parity) {
