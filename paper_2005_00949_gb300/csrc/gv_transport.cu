@@ -1077,7 +1077,7 @@ template <typename R> __device__ __forceinline__ void stage_tables(const DevStat
     sV.zb = zdst;
     sV.inv_node = idst;
     sV.smat = mdst;
-    sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
+    if (S->smax_bytes) sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
     sV.rec = rdst;
   }
   __syncthreads();
@@ -2258,16 +2258,27 @@ template <typename R> int prepare_device(Ctx *c) {
   CK(cudaMalloc(&c->d_state, sizeof(DevState<R>)));
   CK(cudaMalloc(&c->d_part, sizeof(unsigned long long) * (kScanBlocks + 1)));
   CK(cudaMallocHost(&c->h_ctl, sizeof(Ctl)));
-  c->zb_bytes = ((c->nsub + 1) * sizeof(double) + 15) / 16 * 16;
-  c->smax_off = c->xs_bytes + c->zb_bytes + kInvNodeBytes + (c->nsub + 15) / 16 * 16;
-  c->rec_off = c->smax_off + c->smax_bytes;
-  c->req_off = (c->rec_off + c->nsub * sizeof(SubRec<R>) + 31) / 32 * 32;
+  // the integral approach's bound is staged where that approach is on
+  const size_t smax_bytes = (c->cuts.process_mask & GV_P_INTEGRAL) ? c->smax_bytes : 0;
+  const auto layout = [c](size_t smax) {
+    c->smax_bytes = smax;
+    c->zb_bytes = ((c->nsub + 1) * sizeof(double) + 15) / 16 * 16;
+    c->smax_off = c->xs_bytes + c->zb_bytes + kInvNodeBytes + (c->nsub + 15) / 16 * 16;
+    c->rec_off = c->smax_off + smax;
+    c->req_off = (c->rec_off + c->nsub * sizeof(SubRec<R>) + 31) / 32 * 32;
+    c->smem_bytes = c->req_off;
+    if (!c->cfg.pipeline && c->cfg.process_sort)
+      c->smem_bytes += static_cast<size_t>(ReqStore<R>::kBytes) * c->cfg.block_size;
+    c->lk_off = (c->smem_bytes + 31) / 32 * 32;
+    if (!c->cfg.pipeline && c->cfg.process_sort && c->cfg.local_stack)
+      c->smem_bytes = c->lk_off + static_cast<size_t>(LocalStack<R>::kBytes) * c->cfg.block_size;
+  };
+  layout(smax_bytes);
   if (c->cfg.pipeline) {
     const size_t rc_ = static_cast<size_t>(cap);
     if (cudaMalloc(&c->d_req, rc_ * sizeof(GReq<R>)) != cudaSuccess ||
         cudaMalloc(&c->d_keyidx, rc_ * kNReqKey * sizeof(unsigned)) != cudaSuccess)
       return GV_ERR_OOM;
-    c->smem_bytes = c->req_off;
     const void *ka = reinterpret_cast<const void *>(along_kernel<R>);
     const void *kb = reinterpret_cast<const void *>(interact_kernel<R>);
     CK(cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
@@ -2279,14 +2290,25 @@ template <typename R> int prepare_device(Ctx *c) {
     c->grid_b = c->sm_count * occ_b;
     return GV_OK;
   }
-  c->smem_bytes = c->req_off + (c->cfg.process_sort ? static_cast<size_t>(ReqStore<R>::kBytes) * c->cfg.block_size : 0);
-  c->lk_off = (c->smem_bytes + 31) / 32 * 32;
-  if (c->cfg.process_sort && c->cfg.local_stack)
-    c->smem_bytes = c->lk_off + static_cast<size_t>(LocalStack<R>::kBytes) * c->cfg.block_size;
   const void *kern = reinterpret_cast<const void *>(pick_step_kernel<R>(c));
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
   int occ = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, c->cfg.block_size, c->smem_bytes));
+  const auto blocks = [&] {
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, c->cfg.block_size, c->smem_bytes));
+    return static_cast<int>(GV_OK);
+  };
+  if (const int e = blocks()) return e;
+  if (smax_bytes && occ < 2) {
+    // four materials with many sub-slabs: the bound is read from L2 where its
+    // place in shared memory would cost a block
+    const int staged = occ;
+    layout(0);
+    if (const int e = blocks()) return e;
+    if (occ == staged) {
+      layout(smax_bytes);
+      if (const int e = blocks()) return e;
+    }
+  }
   if (occ < 1) return GV_ERR_BAD_ARG;
   c->grid = c->sm_count * std::min(occ, c->cfg.blocks_per_sm);
   return GV_OK;

@@ -1,6 +1,8 @@
 """What surrounds the generations (and the sampler entry point): the prefix sums of the primaries' budgets
 (blocks of 256 primaries each, up to 304 blocks and then longer ranges), and
 tallies accumulated in the caller's buffers or copied to them."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -93,3 +95,26 @@ def test_sampler_kernels_agree_at_their_border(gvmod, model):
     a, b = outs[0][:border - 1], outs[1][:border - 1]
     off = np.abs(a - b) > 1e-6 * np.maximum(np.abs(a), 1e-30)
     assert off.any(axis=1).mean() < 1e-4
+
+
+@pytest.mark.parametrize("integral", [False, True])
+@pytest.mark.parametrize("n_layers", [2, 100, 128])
+def test_histories_do_not_depend_on_where_the_integral_bound_lies(gvmod, integral, n_layers):
+    """With four materials and 800 sub-slabs the bound's place in shared memory
+    costs a block, and it is read from global memory; without the block stack
+    there is room, and with two layers there always is: the same numbers, so
+    equal counts, and deposits up to the order of their FP64 sums."""
+    wl = W.pbps_electrons(200, 500.0)
+    wl = dataclasses.replace(wl, materials=[W.LEAD, W.POLYSTYRENE, W.TUNGSTEN, W.SILICON], n_layers=n_layers,
+                             sub_thick=[0.05, 0.2, 0.02, 0.1, 0.05, 0.1, 0.03, 0.05], sub_mat=[0, 1, 2, 3, 0, 1, 2, 3])
+    if integral:
+        wl = W.with_integral(wl)
+    out = []
+    for kw in (dict(), dict(local_stack=0), dict(block_size=64)):
+        ctx = gvmod.Context(wl, gvmod.gv_default_config(per_event_counts=1, stack_capacity=1 << 18, **kw))
+        out.append(ctx.transport(per_event=True))
+        ctx.close()
+        assert out[-1]["status"] == 0
+    for r in out[1:]:
+        assert np.array_equal(r["counts"][:, :11], out[0]["counts"][:, :11])
+        assert np.abs(r["edep"] - out[0]["edep"]).max() < 1e-9 * 500.0
