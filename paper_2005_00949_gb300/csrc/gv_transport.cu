@@ -401,7 +401,8 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     const R E_pre = t.E;
     // AlongStepAction
     const R Li = pos ? n0.w : n0.z;
-    const Loss<R> loss = loss_at(tab, t.type, t.E, gi, gf, Li, (pos ? n1.w : n1.z) - Li, s, Rr);
+    const R dL = (pos ? n1.w : n1.z) - Li;
+    const Loss<R> loss = loss_at(tab, t.type, t.E, gi, gf, Li, dL, loss_slope(n0, t.type, dL), s, Rr);
     const R Ep = loss_energy(loss);
     deposit<R, EXT>(S, edep, t.ev, pre_sub, mx, my, t.E - Ep, pd);
     t.E = Ep;
@@ -2050,6 +2051,9 @@ template <typename R> int upload_tables(Ctx *c) {
     xs[i].z = static_cast<R>(type == 1 ? std::log(h.xs[4 * i + 2]) : h.xs[4 * i + 2]);
     xs[i].w = static_cast<R>(type == 2 ? std::log(h.xs[4 * i + 3]) : h.xs[4 * i + 3]);
   }
+  if (sizeof(R) == 8)  // an electron's free component: the slope of its ln R (loss_slope)
+    for (size_t i = 0; i + 1 < nv; ++i)
+      if ((i / kGridN) % 3 == 1 && i % kGridN + 1 < kGridN) xs[i].w = static_cast<R>(kLnNode / (xs[i + 1].z - xs[i].z));
   c->xs_bytes = nv * sizeof(V4<R>);
   CK(cudaMalloc(&c->d_xs, c->xs_bytes));
   CK(cudaMemcpy(c->d_xs, xs.data(), c->xs_bytes, cudaMemcpyHostToDevice));

@@ -35,7 +35,7 @@ __global__ void k_lookup(View<R> V, int type, int mat, const double *E, long lon
   out[4 * i] = v.x;
   out[4 * i + 1] = v.y;
   out[4 * i + 2] = type == 1 ? range_of(v, type) : v.z;  // the range, from its interpolated logarithm
-  out[4 * i + 3] = type == 2 ? range_of(v, type) : v.w;
+  out[4 * i + 3] = type == 2 ? range_of(v, type) : (type == 1 ? R(0) : v.w);
 }
 
 template <typename R>
