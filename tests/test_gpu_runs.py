@@ -5,6 +5,7 @@ subtracting coordinates, so backward, oblique, lateral and on-plane starts are
 run with one step per run (every distance from coordinates) and with long
 runs.  With one step per run against many the same FP32 operations are done:
 integer counts are equal and deposits differ by the order of the FP64 sums."""
+import dataclasses
 import os
 
 import numpy as np
@@ -103,3 +104,25 @@ def test_field_too_weak_to_turn_a_step(precision, tesla):
     eps = 2.0 ** (-22 if precision == 0 else -51)
     assert (np.abs(g[:, :3] - s[:, None] * d) <= eps * s[:, None] + tesla * s[:, None] ** 2).all()
     assert (np.abs(g[:, 3:6] - d) <= eps + tesla * s[:, None]).all()
+
+
+@pytest.mark.parametrize("thick, mat", [([0.2, 0.2, 0.5], [0, 1, 0]), ([0.3, 0.1, 0.1], [0, 0, 1]), ([0.4], [1])])
+def test_fp64_runs_across_repeated_slabs(thick, mat):
+    """An FP64 photon run takes cross sections and paths over from the
+    sub-slab before the last where table row or thickness are the same: each
+    may repeat without the other, and in a stack of one kind always.  One step
+    a run takes nothing over, and gives the same histories."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    wl = dataclasses.replace(_both_ways(), n_layers=50, sub_thick=thick, sub_mat=mat)
+    out = []
+    for budget in (1, 64):
+        ctx = gv.Context(wl, gv.gv_default_config(precision=1, per_event_counts=1, stack_capacity=1 << 20,
+                                                  along_steps=budget, along_steps_photon=budget))
+        out.append(ctx.transport(per_event=True))
+        ctx.close()
+        assert out[-1]["status"] == 0
+    assert np.array_equal(out[0]["counts"][:, :11], out[1]["counts"][:, :11])
+    assert np.abs(out[0]["edep"] - out[1]["edep"]).max() < 1e-9 * 400.0
+    assert np.abs(out[0]["escape"] - out[1]["escape"]).max() < 1e-9 * 400.0
