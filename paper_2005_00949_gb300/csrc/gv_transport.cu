@@ -793,139 +793,118 @@ template <typename R> struct LocalStack {
   }
 };
 
-// PostStepActions: append the step's secondaries to the output queues, or,
-// with a local stack, to the block's stack while it has room.  Called by all
-// 32 lanes of a converged warp (lanes without secondaries pass kids.n == 0).
-template <typename R, bool EXT = true>
-__device__ __forceinline__ void push_kids(const DevState<R> *S, int out, const Parent &t, const Kids<R> &kids,
-                                          uint32_t kk, const uint4 &ids, unsigned long long *row,
-                                          const LocalStack<R> *ls = nullptr) {
-  const unsigned b0 = __ballot_sync(0xffffffffu, kids.n > 0);
-  if (!b0) return;
+// A lane's running count in a warp: the sum over its own and the lower lanes.
+__device__ __forceinline__ unsigned lane_sum(unsigned v) {
   const int lane = threadIdx.x & 31;
-  uint32_t w[6] = {0, 0, 0, 0, 0, 0};
-  if (kids.n > 0) {
-    w[0] = ids.x; w[1] = ids.y; w[2] = ids.z; w[3] = ids.w;
-    if (kids.n > 2) {
-      const uint4 b = track_draw(S, t.id, t.ev, kk, kTagId + 1u);
-      w[4] = b.x; w[5] = b.y;
-    }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
   }
-  const unsigned b1 = __ballot_sync(0xffffffffu, kids.n > 1);
-  const unsigned b2 = __ballot_sync(0xffffffffu, kids.n > 2);
-  // the block's stack first, while it has room (the ids above keep each
-  // kid's index in the list, so where it goes changes no result)
-  int room = 0;  // the lane's first `room` kids go to the block's stack
-  if (ls) {
-    // the warp's kids in order: lane by lane, within a lane by index
-    unsigned mg[3], mq[3];  // lanes whose kid j is a photon, a charged track
-    unsigned ng = 0, nq = 0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      mg[j] = __ballot_sync(0xffffffffu, j < kids.n && kids.type[j] == 0);
-      mq[j] = __ballot_sync(0xffffffffu, j < kids.n && kids.type[j] != 0);
-      ng += __popc(mg[j]);
-      nq += __popc(mq[j]);
-    }
-    const unsigned lt = (1u << lane) - 1u;
-    const unsigned before = __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt);
-    unsigned used = 0;
-    if (lane == 0) used = atomicAdd(&ls->count->used, ng | nq << 16);
-    used = __shfl_sync(0xffffffffu, used, 0);
-    const int free = ls->cap - static_cast<int>((used & 0xffffu) + (used >> 16));
-    room = max(0, min(free - static_cast<int>(before), kids.n));
-    unsigned g = (used & 0xffffu) + __popc(mg[0] & lt) + __popc(mg[1] & lt) + __popc(mg[2] & lt);
-    unsigned q = (used >> 16) + __popc(mq[0] & lt) + __popc(mq[1] & lt) + __popc(mq[2] & lt);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (j >= kids.n) continue;
-      const int charged = kids.type[j] != 0;
-      if (j < room)
-        ls->put(ls->place(charged, charged ? q : g), t,
-                static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
-                kids.d[j], kids.E[j], kids.type[j]);
-      q += charged;
-      g += 1 - charged;
-    }
-    if (static_cast<int>(ng + nq) > free) {  // uniform: take back what did not fit
-      unsigned back = 0;
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        if (j < kids.n && j >= room) back += kids.type[j] == 0 ? 1u : 1u << 16;
-      back = __reduce_add_sync(0xffffffffu, back);
-      if (lane == 0) atomicSub(&ls->count->used, back);
-    }
+  return v;
+}
+
+// The ids of a final state's secondaries are words of counter blocks of its
+// step (ids: the first two's), so they name each one's index in its parent's
+// list, and where it goes changes no result.
+template <typename R>
+__device__ __forceinline__ unsigned long long kid_id(const DevState<R> *S, const Parent &p, uint32_t kk, const uint4 &ids, int j) {
+  uint32_t lo = j ? ids.z : ids.x, hi = j ? ids.w : ids.y;
+  if (j == 2) {
+    const uint4 b = track_draw(S, p.id, p.ev, kk, kTagId + 1u);
+    lo = b.x; hi = b.y;
   }
-  WarpAppend ap, all;
-  unsigned rank[3] = {0, 0, 0};
-  const unsigned bj[3] = {b0, b1, b2};
+  return static_cast<unsigned long long>(lo) | (static_cast<unsigned long long>(hi) << 32);
+}
+
+// Put the secondaries of a warp's final states on the block's stack while it
+// has room.  Returns how many of the lane's the stack took; what it refuses
+// leaves it exactly full, so that no later reservation of the round finds
+// room.  All 32 lanes of a converged warp.
+template <typename R, bool EXT = true>
+__device__ __forceinline__ int stack_kids(const DevState<R> *S, const LocalStack<R> &ls, const Parent &p, const Kids<R> &kids,
+                                          uint32_t kk, const uint4 &ids, unsigned long long *row) {
+  if (!__any_sync(0xffffffffu, kids.n > 0)) return 0;
+  const int lane = threadIdx.x & 31;
+  // photons | charged tracks << 16: the lane's, up to it, and the warp's
+  unsigned mine = 0u;
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    if (j < kids.n) mine += kids.type[j] == 0 ? 1u : 1u << 16;
+  const unsigned incl = lane_sum(mine);
+  const unsigned all = __shfl_sync(0xffffffffu, incl, 31);
+  unsigned used = 0;
+  if (lane == 0) used = atomicAdd(&ls.count->used, all);
+  used = __shfl_sync(0xffffffffu, used, 0);
+  const int free = ls.cap - static_cast<int>((used & 0xffffu) + (used >> 16));
+  const unsigned before = incl - mine;
+  const int room = max(0, min(free - static_cast<int>((before & 0xffffu) + (before >> 16)), kids.n));
+  unsigned at = used + before, made = 0u;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    if (!bj[j]) continue;
-    if (ls) all.add(j < kids.n, kids.type[j]);
-    rank[j] = ap.add(j < kids.n && j >= room, kids.type[j]);
+    if (j >= room) break;
+    const int charged = kids.type[j] != 0;
+    ls.put(ls.place(charged, charged ? at >> 16 : at & 0xffffu), p, kid_id(S, p, kk, ids, j), kids.d[j], kids.E[j],
+           kids.type[j]);
+    at += charged ? 1u << 16 : 1u;
+    made += 1u << 8 * kids.type[j];
+    if (EXT && S->evcnt) atomicAdd(&S->evcnt[static_cast<size_t>(p.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
   }
+  if (static_cast<int>((all & 0xffffu) + (all >> 16)) > free) {  // uniform: take back what did not fit
+    const unsigned back = __reduce_add_sync(0xffffffffu, used + incl - at);
+    if (lane == 0) atomicSub(&ls.count->used, back);
+  }
+  made = __reduce_add_sync(0xffffffffu, made);
+  if (lane >= GV_C_TRK_G && lane < GV_C_TRK_G + 3) row[lane] += made >> 8 * (lane - GV_C_TRK_G) & 0xffu;
+  return room;
+}
+
+// The end of a claim: the secondaries of the final states the warp ran, from
+// `first` on (the block's stack took the others; t's are its own), and its
+// lanes' survivors, appended with one reservation: a trip to L2 less per
+// claim, and the block does not wait at the results barrier for the warps that
+// append secondaries (2000 x 10 GeV: 4.16 -> 3.99 ms).  What bounds it is its
+// length: a warp comes here once per claim and fetches most of the
+// instructions anew (ballots and ranks record by record took 3500 cycles of a
+// claim's 19000, unloaded as well).  So one sum over the lanes, of the records
+// of each type a byte each, gives all ranks and counts, and every round's
+// appends share this site: the kernel 110 -> 104 KB, 3.99 -> 3.88 ms, 4096
+// mixed 10.88 -> 10.62 ms, 1000 x 1 GeV 720 -> 704 us.  All 32 lanes of a
+// converged warp.
+template <typename R, bool EXT = true>
+__device__ __forceinline__ void push_all(const DevState<R> *S, int out, const Parent &p, const Kids<R> &kids, int first,
+                                         const uint4 &ids, uint32_t kk, const Trk<R> &t, bool alive,
+                                         unsigned long long *row) {
+  const int lane = threadIdx.x & 31;
+  // the lane's records per type, a byte each (a warp has 128 at most)
+  unsigned made = 0u;
 #pragma unroll
-  for (int q = 0; q < 3; ++q) wcnt_add(row, GV_C_TRK_G + q, ls ? all.n[q] : ap.n[q]);
+  for (int j = 0; j < 3; ++j)
+    if (j >= first && j < kids.n) made += 1u << 8 * kids.type[j];
+  const unsigned mine = made + (alive ? 1u << 8 * t.type : 0u);
+  unsigned at = lane_sum(mine);
+  const unsigned all = __shfl_sync(0xffffffffu, at, 31);
+  const unsigned n = lane < 3 ? all >> 8 * lane & 0xffu : 0u;
+  const unsigned base = n ? atomicAdd(&S->ctl->cnt[out][lane].n, n) : 0u;
+  made = __reduce_add_sync(0xffffffffu, made);
+  if (lane >= GV_C_TRK_G && lane < GV_C_TRK_G + 3) row[lane] += made >> 8 * (lane - GV_C_TRK_G) & 0xffu;
   if (EXT && S->evcnt) {
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      if (j < kids.n) atomicAdd(&S->evcnt[static_cast<size_t>(t.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
+      if (j >= first && j < kids.n)
+        atomicAdd(&S->evcnt[static_cast<size_t>(p.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
   }
-  if (!(ap.n[0] | ap.n[1] | ap.n[2])) return;
-  const unsigned base = ap.reserve(S->ctl->cnt[out]);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    if (!bj[j]) continue;
-    const bool has = j < kids.n && j >= room;
-    const unsigned slot = WarpAppend::slot(base, has ? kids.type[j] : 0, rank[j]);
-    if (!has) continue;
-    if (slot >= S->capacity) {
-      set_status(S->ctl, GV_ERR_STACK_FULL);
-      continue;
-    }
-    store_track<R>(S, out, kids.type[j], slot, t.x, t.y, t.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j],
-                   R(-1), static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
-                   t.ev, 0u, t.sub);
-  }
-}
-
-// The end of a claim: the secondaries of the final states the warp ran (t's
-// are its own) and its lanes' survivors, appended with one reservation: a trip
-// to L2 less per claim, and the block does not wait at the results barrier for
-// the warps that append secondaries (2000 x 10 GeV: 4.16 -> 3.99 ms).  All 32
-// lanes of a converged warp.
-template <typename R, bool EXT = true>
-__device__ __forceinline__ void push_all(const DevState<R> *S, int out, const Parent &p, const Kids<R> &kids,
-                                         const uint4 &ids, uint32_t kk, const Trk<R> &t, bool alive,
-                                         unsigned long long *row) {
-  uint32_t w[6] = {ids.x, ids.y, ids.z, ids.w, 0u, 0u};
-  if (kids.n > 2) {
-    const uint4 b = track_draw(S, p.id, p.ev, kk, kTagId + 1u);
-    w[4] = b.x; w[5] = b.y;
-  }
-  WarpAppend ap;
-  unsigned rank[3] = {0, 0, 0};
-  bool some[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    some[j] = __any_sync(0xffffffffu, j < kids.n);
-    if (some[j]) rank[j] = ap.add(j < kids.n, kids.type[j]);
-  }
-  if (some[0]) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) wcnt_add(row, GV_C_TRK_G + q, ap.n[q]);
-    if (EXT && S->evcnt) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        if (j < kids.n) atomicAdd(&S->evcnt[static_cast<size_t>(p.ev) * GV_NCOUNT + GV_C_TRK_G + kids.type[j]], 1ull);
-    }
-  }
-  const unsigned srank = ap.add(alive, t.type);
-  const unsigned base = ap.reserve(S->ctl->cnt[out]);
-  const unsigned slot = WarpAppend::slot(base, alive ? t.type : 0, srank);
+  at -= mine;
+  const unsigned b0 = __shfl_sync(0xffffffffu, base, 0), b1 = __shfl_sync(0xffffffffu, base, 1),
+                 b2 = __shfl_sync(0xffffffffu, base, 2);
   bool full = false;
+  const auto place = [&](int type) {
+    const unsigned slot = (type == 0 ? b0 : (type == 1 ? b1 : b2)) + (at >> 8 * type & 0xffu);
+    at += 1u << 8 * type;
+    return slot;
+  };
   if (alive) {
+    const unsigned slot = place(t.type);
     if (slot < S->capacity)
       store_track<R>(S, out, t.type, slot, t.x, t.y, t.z, t.u, t.v, t.w, t.E, t.nlam, t.id, t.ev, t.step,
                      t.sub | (t.flags << 16));
@@ -933,17 +912,26 @@ __device__ __forceinline__ void push_all(const DevState<R> *S, int out, const Pa
   }
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    if (!some[j]) continue;
-    const bool has = j < kids.n;
-    const unsigned ks = WarpAppend::slot(base, has ? kids.type[j] : 0, rank[j]);
-    if (!has) continue;
-    if (ks < S->capacity)
-      store_track<R>(S, out, kids.type[j], ks, p.x, p.y, p.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j], R(-1),
-                     static_cast<unsigned long long>(w[2 * j]) | (static_cast<unsigned long long>(w[2 * j + 1]) << 32),
-                     p.ev, 0u, p.sub);
+    if (j < first || j >= kids.n) continue;
+    const unsigned slot = place(kids.type[j]);
+    if (slot < S->capacity)
+      store_track<R>(S, out, kids.type[j], slot, p.x, p.y, p.z, kids.d[j][0], kids.d[j][1], kids.d[j][2], kids.E[j], R(-1),
+                     kid_id(S, p, kk, ids, j), p.ev, 0u, p.sub);
     else full = true;
   }
   if (full) set_status(S->ctl, GV_ERR_STACK_FULL);
+}
+
+// PostStepActions: append the step's secondaries to the output queues.
+// Called by all 32 lanes of a converged warp (lanes without secondaries pass
+// kids.n == 0).
+template <typename R, bool EXT = true>
+__device__ __forceinline__ void push_kids(const DevState<R> *S, int out, const Parent &t, const Kids<R> &kids,
+                                          uint32_t kk, const uint4 &ids, unsigned long long *row) {
+  if (!__any_sync(0xffffffffu, kids.n > 0)) return;
+  Trk<R> none;
+  none.type = 0;
+  push_all<R, EXT>(S, out, t, kids, 0, ids, kk, none, false, row);
 }
 
 // Survivors: one record per lane (has: whether it has one).  All 32 lanes of
@@ -1669,6 +1657,7 @@ __global__ void GV_STEP_BOUNDS
       Parent par;
       uint32_t pk = 0;
       uint4 ids = make_uint4(0u, 0u, 0u, 0u);
+      int first = 0;  // of the lane's secondaries, the first that is not on the stack
       {
         int np = 0, na = 0;
         if (static_cast<unsigned>(tid) < nreq) {
@@ -1693,9 +1682,8 @@ __global__ void GV_STEP_BOUNDS
         }
         wcnt_add(row, GV_C_PAIR, __popc(__ballot_sync(0xffffffffu, np)));
         wcnt_add(row, GV_C_ANNIH, __popc(__ballot_sync(0xffffffffu, na)));
-        // with more rounds to come the secondaries go out (or on the stack) now;
-        // the last round's wait for the survivors
-        if (kk + 1 < K) push_kids<R, EXT>(S, out, par, kb, pk, ids, row, use_local ? &lstk : nullptr);
+        // with more rounds to come the secondaries go on the block's stack
+        if (use_local && kk + 1 < K) first = stack_kids<R, EXT>(S, lstk, par, kb, pk, ids, row);
       }
       __syncthreads();
       if (key >= 0 && key != kKeyRest) {
@@ -1712,8 +1700,9 @@ __global__ void GV_STEP_BOUNDS
         // the next claim's atomic is in flight while the claim's tracks go out
         if (tid == 0) next_chunk = gridDim.x + atomicAdd(&ctl->claim.n, 1u);
         claimed = true;
-        push_all<R, EXT>(S, out, par, kb, ids, pk, t, alive, row);
       }
+      if (kk + 1 == K || __any_sync(0xffffffffu, first < kb.n))
+        push_all<R, EXT>(S, out, par, kb, first, ids, pk, t, alive && kk + 1 == K, row);
       // (the event counts' atomics were in flight while the tracks went out)
       if (ended_own == 1u) event_closed(S, t.ev);
       if (ended_req == 1u) event_closed(S, ev_req);

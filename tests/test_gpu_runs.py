@@ -126,3 +126,25 @@ def test_fp64_runs_across_repeated_slabs(thick, mat):
     assert np.array_equal(out[0]["counts"][:, :11], out[1]["counts"][:, :11])
     assert np.abs(out[0]["edep"] - out[1]["edep"]).max() < 1e-9 * 400.0
     assert np.abs(out[0]["escape"] - out[1]["escape"]).max() < 1e-9 * 400.0
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("block", [64, 256])
+def test_a_full_block_stack_loses_no_secondary(prec, block):
+    """Blocks of charged tracks with long claims make more secondaries a round
+    than their stacks hold, so reservations are refused all the time, several
+    at once in the larger block: histories stay those without a stack."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    wl = W.pbps_electrons(40_000 if prec == 0 else 8_000, 60.0)
+    out = []
+    for kw in (dict(local_stack=0, tail_steps_per_claim=1), dict(tail_steps_per_claim=16, tail_threshold=1 << 40)):
+        ctx = gv.Context(wl, gv.gv_default_config(precision=prec, per_event_counts=1, block_size=block,
+                                                  stack_capacity=1 << 20, **kw))
+        for _ in range(3):
+            out.append(ctx.transport(per_event=True))
+            assert out[-1]["status"] == 0, kw
+            assert np.array_equal(out[-1]["counts"][:, :11], out[0]["counts"][:, :11]), kw
+            assert np.abs(out[-1]["edep"] - out[0]["edep"]).max() < 1e-9 * 60.0, kw
+        ctx.close()
