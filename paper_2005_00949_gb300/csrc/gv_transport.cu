@@ -567,17 +567,19 @@ __device__ __forceinline__ int final_state(const View<R> &V, const DevState<R> *
   ids = track_draw(S, id, ev, kk, kTagId);
   const R u[8] = {R(0), R(0), u2, u3, u24<R>(r1.x), u24<R>(r1.y), u24<R>(r1.z), u24<R>(r1.w)};
   int r = 0;
-  if (key == kKeyRest) {
-    at_rest(kids, u[6], u[7]);
-    na = 1;
-  } else {
+  bool rest = key == kKeyRest;
+  if (!rest) {
     const int type = key / 3;
     R local;
     const RngKey g = {static_cast<uint32_t>(id), static_cast<uint32_t>(id >> 32), kk, S->seed_lo ^ (ev + S->ev_base),
                       S->seed_hi};
-    r = interact<R, OPTS, ALT>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na);
+    r = interact<R, OPTS, ALT>(V, type, key - 3 * type, E, d, u, g, kids, local, np, na, rest);
     if (r < 0) return -1;
     deposit<R, EXT>(S, S->edep + static_cast<size_t>(ev) * S->view.geo.nsub, ev, sub, x, y, local, pd);
+  }
+  if (rest) {  // a stopped positron, of this final state or of the run
+    at_rest(kids, u[6], u[7]);
+    na += 1;
   }
   if (EXT && S->evcnt) {
     unsigned long long *row = &S->evcnt[static_cast<size_t>(ev) * GV_NCOUNT];

@@ -71,7 +71,9 @@ __global__ void k_interact(View<R> V, int type, int proc, const double *E, const
   int np = 0, na = 0;
   // a rejection sampler, where configured, draws from the stream (i, 0, 0) under key (0, 0)
   const RngKey g = {static_cast<uint32_t>(i), static_cast<uint32_t>(i >> 32), 0u, 0u, 0u};
-  const int r = interact(V, type, proc, e, d, uu, g, kids, local, np, na);
+  bool rest = false;
+  const int r = interact(V, type, proc, e, d, uu, g, kids, local, np, na, rest);
+  if (rest) at_rest(kids, uu[6], uu[7]);
   double *o = out + 24 * i;
   for (int j = 0; j < 24; ++j) o[j] = 0.0;
   o[0] = r == 1 ? static_cast<double>(e) : (r == 0 ? -1.0 : E[i]);
