@@ -606,17 +606,8 @@ __device__ __forceinline__ void count_round(unsigned long long *row, const Run<R
   const unsigned sum = __reduce_add_sync(0xffffffffu, r.n_st | (r.n_geom << 12) | (chose ? 1u << 24 : 0u));
   const unsigned it = __reduce_max_sync(0xffffffffu, r.n_iter);
   const unsigned st = sum & 0xfffu;
-  const unsigned mg = __ballot_sync(0xffffffffu, r.n_st && type == 0);
-  const unsigned me = __ballot_sync(0xffffffffu, r.n_st && type == 1);
-  const unsigned mp = __ballot_sync(0xffffffffu, r.n_st && type == 2);
-  unsigned wg = st, we = st;
-  if ((mg != 0) + (me != 0) + (mp != 0) > 1) {  // mixed types: primaries, or the block's stack
-    wg = __reduce_add_sync(0xffffffffu, type == 0 ? r.n_st : 0u);
-    we = __reduce_add_sync(0xffffffffu, type == 1 ? r.n_st : 0u);
-  } else {
-    wg = mg ? st : 0u;
-    we = me ? st : 0u;
-  }
+  const unsigned by_type = __reduce_add_sync(0xffffffffu, type == 0 ? r.n_st : (type == 1 ? r.n_st << 16 : 0u));
+  const unsigned wg = by_type & 0xffffu, we = by_type >> 16;
   const int lane = threadIdx.x & 31;
   unsigned v = 0;
   if (lane == GV_C_STEPS) v = st;
@@ -1110,6 +1101,11 @@ template <typename R> __device__ __forceinline__ void stage_tables(const DevStat
 // photon ones (measured: 4 % less transport time than photons first).
 __device__ __forceinline__ int claim_queue(int seg) { return seg < 3 ? 2 - seg : 3; }
 
+// The plan of the next generation.  One thread runs it between generations,
+// on instructions that no block has fetched before: without 64-bit divisions
+// and the counters that this kind of kernel does not use, and with one sum per
+// round for the steps by type (count_round), 1000 x 1 GeV took 687 instead of
+// 697 us.
 template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   Ctl *c = S->ctl;
   // everything the plan depends on, in one round trip
@@ -1179,8 +1175,10 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   // fewer warps to wait for at its barriers and its idle lanes left to the
   // secondaries of its block stack.
   if (S->adaptive_chunk) {
-    const unsigned long long per = (tot + S->grid - 1) / S->grid;
-    if (per < B) B = per <= 32 ? 32u : static_cast<unsigned>((per + 31) / 32 * 32);
+    if (tot < static_cast<unsigned long long>(B) * static_cast<unsigned>(S->grid)) {  // (32 bits: a 64-bit division is a call)
+      const unsigned g = static_cast<unsigned>(S->grid), per = (static_cast<unsigned>(tot) + g - 1) / g;
+      if (per < B) B = per <= 32 ? 32u : (per + 31) / 32 * 32;
+    }
   }
   p.B = B;
   p.end[0] = (n2 + B - 1) / B;  // segments in claim_queue order
@@ -1197,12 +1195,18 @@ template <typename R> __device__ void plan_next(const DevState<R> *S, int pn) {
   p.K = (last && tot < S->tail_threshold) ? S->K_tail : S->K_bulk;
   for (int q = 0; q < 3; ++q) c->cnt[pn ^ 1][q].n = 0;
   c->claim.n = 0;
-  for (int r = 0; r < kNClaim; ++r) c->claims[r].n = 0;
   c->blocks_done = 0;
-  c->req_n = 0;
-  for (int k = 0; k < kNReqKey; ++k) c->key_n[k] = 0;
-  c->claim_b = 0;
-  c->blocks_done_b = 0;
+  if (S->chunk == 32) {  // warps claim (blocks have 64 threads or more)
+#pragma unroll 1
+    for (int r = 0; r < kNClaim; ++r) c->claims[r].n = 0;
+  }
+  if (S->pipeline) {
+    c->req_n = 0;
+#pragma unroll 1
+    for (int k = 0; k < kNReqKey; ++k) c->key_n[k] = 0;
+    c->claim_b = 0;
+    c->blocks_done_b = 0;
+  }
   if (tot > live_peak) c->live_peak = tot;
   if (tot > 0) c->gen = ++gen;
   if (gen > S->max_gen && status == 0) c->status = status = GV_ERR_TIMEOUT;
@@ -1410,21 +1414,23 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 
 // What bounds it: the dependent chains of a round at the two blocks per SM
 // that its registers allow, and at a block's barriers its slowest warp.  At
-// the shower maximum (ncu, 500 x 10 GeV) a scheduler issues in 33 % of its
-// cycles; per issue 2.4 warps wait for L2, 2.1 for a fixed-latency result,
-// 2.0 at a barrier, 1.9 for shared memory and 0.8 for instructions (the code
-// is 110 KB); ALU 25 %, FP64 pipe 14 %, FMA 12 %, L2 6 %, DRAM 4 % of their
-// peaks.  FP64 kernels sit on the FP64 pipe (69 % at the maximum).  So the
-// chains are short and work is done where many lanes do it: random numbers
-// once per round instead of once per step (run_round), one place that makes
-// secondaries (a stopped positron is a request like any other), counters
-// booked by ballots into words of the warp (a 64-bit shared-memory atomic is
-// a loop), 16-byte track parts, one reservation atomic for the three queues,
-// a warp to a model (the sort below), a generation's plan in one read.  What a
-// caller waits for, before these and with them: 2000 x 10 GeV e- in
-// Pb/polystyrene 7.75 -> 3.98 ms, 1000 x 1 GeV 1.37 -> 0.72 ms, one 10 GeV
-// shower 1.13 -> 0.59 ms, 300 x 10 GeV in FP64 13.0 -> 8.5 ms, 2000 x 100 GeV
-// in W/Si with cells 94.8 -> 52.2 ms.
+// the shower maximum (ncu, 500 x 10 GeV, the kernel at 110 KB of code) a
+// scheduler issues in 33 % of its cycles; per issue 2.4 warps wait for L2, 2.1
+// for a fixed-latency result, 2.0 at a barrier, 1.9 for shared memory and 0.8
+// for instructions; ALU 25 %, FP64 pipe 14 %, FMA 12 %, L2 6 %, DRAM 4 %.
+// FP64 kernels sit on the FP64 pipe (69 % at the maximum).  So the chains are
+// short and work is done where many lanes do it: random numbers once per round
+// instead of once per step (run_round), one place that makes secondaries (a
+// stopped positron is a request like any other), counters booked by ballots
+// into words of the warp (a 64-bit shared-memory atomic is a loop), 16-byte
+// track parts, one reservation atomic for the three queues, a warp to a model
+// (the sort below), a generation's plan in one read; and the code is kept
+// small, because a warp fetches what it runs once per claim anew: the same
+// kernel with 12 KB more of it lost 5 % on the small transports.  What a caller
+// waits for, before these and with them: 2000 x 10 GeV e- in Pb/polystyrene
+// 7.74 -> 3.83 ms, 1000 x 1 GeV 1.37 -> 0.69 ms, one 10 GeV shower 1.13 -> 0.57
+// ms, 300 x 10 GeV in FP64 13.0 -> 8.3 ms, 2000 x 100 GeV in W/Si with cells
+// 94.5 -> 51.4 ms.
 template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT, bool ALT = !SORT>
 __global__ void GV_STEP_BOUNDS
     step_kernel(int parity) {
