@@ -1414,10 +1414,10 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 
 // What bounds it: the dependent chains of a round at the two blocks per SM
 // that its registers allow, and at a block's barriers its slowest warp.  At
-// the shower maximum (ncu, 500 x 10 GeV, the kernel at 110 KB of code) a
-// scheduler issues in 33 % of its cycles; per issue 2.4 warps wait for L2, 2.1
-// for a fixed-latency result, 2.0 at a barrier, 1.9 for shared memory and 0.8
-// for instructions; ALU 25 %, FP64 pipe 14 %, FMA 12 %, L2 6 %, DRAM 4 %.
+// the shower maximum (ncu, 500 x 10 GeV) a scheduler issues in 34 % of its
+// cycles; per issue 2.4 warps wait for L2, 2.1 for a fixed-latency result, 1.9
+// for shared memory, 1.8 at a barrier and 0.7 for instructions; ALU 26 %, FP64
+// pipe 15 %, FMA 13 %, L2 7 %, DRAM 4 % of their peaks.
 // FP64 kernels sit on the FP64 pipe (69 % at the maximum).  So the chains are
 // short and work is done where many lanes do it: random numbers once per round
 // instead of once per step (run_round), one place that makes secondaries (a
