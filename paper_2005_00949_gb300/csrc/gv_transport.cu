@@ -1449,7 +1449,11 @@ __global__ void GV_STEP_BOUNDS
   // start as soon as this one's finish, stage their tables, and wait for
   // this grid (and its plan) to complete before reading the plan.
   asm volatile("griddepcontrol.launch_dependents;");
-  if (ctl->plan.done) return;  // a done flag seen before the wait is final: nothing planned
+  // A done flag seen before the wait is final: nothing is planned, and the block
+  // leaves.  The previous generation may set it while the block looks, so one
+  // verdict holds for the block: what its threads do after the wait (the plan
+  // is read by sixteen of them) is done by all of them or by none.
+  if (__syncthreads_or(ctl->plan.done)) return;
   unsigned long long *const row = s_wc[tid >> 5];
   if (lane < 16) row[lane] = 0ull;
   if (tid < 2 * kNKey) s_key[tid / kNKey][tid % kNKey] = 0u;
