@@ -338,6 +338,9 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
   // soon as z is known, and it is done when the loss is
   R s_geom = t.w != R(0) ? by_w.div(dz) : INF;
   walls(geo, t.x, t.y, t.u, t.v, lat, s_geom, wall);
+  // the wall that the pre-step direction points at (-4, -5: the lower one): a
+  // field may turn the track within the step
+  if (wall < -1 && !((wall == -2 ? t.u : t.v) > R(0))) wall -= 2;
   if (s_geom < R(0)) s_geom = R(0);
   int m = 0, end = kRunOn;
   for (;;) {
@@ -436,6 +439,11 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     t.E = Ep;
     ++m;
     if (t.E < tcut) {
+      if (lim == 0 && wall < -1) {  // it stops on the wall
+        const double w = wall == -2 ? geo.wx[1] : (wall == -4 ? geo.wx[0] : (wall == -3 ? geo.wy[1] : geo.wy[0]));
+        if (wall & 1) t.y = w;
+        else t.x = w;
+      }
       deposit<R, EXT>(S, edep, t.ev, pre_sub, t.x, t.y, t.E, pd);
       end = t.type == 2 ? kRunRest : kRunEnd;
       break;
@@ -468,10 +476,6 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     if (!walls_clear(lat, s_geom)) break;
     if (s_geom < R(0)) s_geom = R(0);
     wall = -1;
-  }
-  if (wall < -1 && lim == 0) {  // a step to a wall ends on it
-    if (wall == -2) t.x = t.u > R(0) ? geo.wx[1] : geo.wx[0];
-    else t.y = t.v > R(0) ? geo.wy[1] : geo.wy[0];
   }
   return end;
 }
