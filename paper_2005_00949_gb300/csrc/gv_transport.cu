@@ -2280,6 +2280,22 @@ template <typename R> class StateSlot {
   cudaEvent_t ev_;
 };
 
+// Lets launches of `kern` on the current device have `bytes` of dynamic shared
+// memory.  The limit is a property of the function, which contexts of other
+// sizes and other threads launch too (or have captured and launch later), so
+// it is always raised to the same value, the most a block of this kernel can
+// have, and never lowered to what one of them needs.
+cudaError_t allow_shared(const void *kern, int device, size_t bytes) {
+  cudaFuncAttributes a;
+  int most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&a, kern);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  if (e != cudaSuccess) return e;
+  most -= static_cast<int>(a.sharedSizeBytes);
+  if (most < 0 || bytes > static_cast<size_t>(most)) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 template <typename R> int prepare_device(Ctx *c) {
   CK(cudaSetDevice(c->device));
   CK(slot_event_create(c->device, sizeof(R) == 8));
@@ -2318,7 +2334,7 @@ template <typename R> int prepare_device(Ctx *c) {
       return GV_ERR_OOM;
     const void *ka = reinterpret_cast<const void *>(along_kernel<R>);
     const void *kb = reinterpret_cast<const void *>(interact_kernel<R>);
-    CK(cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
+    CK(allow_shared(ka, c->device, c->smem_bytes));
     int occ = 0, occ_b = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ka, c->cfg.block_size, c->smem_bytes));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b, kb, 256, 0));
@@ -2330,7 +2346,7 @@ template <typename R> int prepare_device(Ctx *c) {
   const void *kern = reinterpret_cast<const void *>(pick_step_kernel<R>(c));
   int occ = 0;
   const auto blocks = [&] {
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(c->smem_bytes)));
+    CK(allow_shared(kern, c->device, c->smem_bytes));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, c->cfg.block_size, c->smem_bytes));
     return static_cast<int>(GV_OK);
   };
@@ -3043,9 +3059,7 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
   const int block = c->cfg.block_size;
   const size_t lk_off = (c->req_off + static_cast<size_t>(ReqStore<float>::kBytes) * block + 31) / 32 * 32;
   const size_t smem = lk_off + static_cast<size_t>(LocalStack<float>::kBytes) * block;
-  if (cudaFuncSetAttribute(reinterpret_cast<const void *>(step), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess)
-    return GV_ERR_CUDA;
+  if (allow_shared(reinterpret_cast<const void *>(step), c->device, smem) != cudaSuccess) return GV_ERR_CUDA;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, reinterpret_cast<const void *>(step), block, smem) != cudaSuccess ||
       occ < 1)
