@@ -184,6 +184,10 @@ constexpr int kTabThreads = 1024;
 // 2^18 samples take 8.1 us this way and 7.6 us through L1, 2^19 10.1 and
 // 9.9, 2^20 13.4 and 14.6, 2^22 37 and 45 (the mean of three models' tables).
 constexpr long long kTabMin = 1 << 20;
+// The rows must leave room for two blocks on an SM.  It is also what the
+// kernel's limit of dynamic shared memory is set to, whatever the model: the
+// limit belongs to the function, and threads sample different models at once.
+constexpr size_t kTabBytes = 100 * 1024;
 
 __global__ void __launch_bounds__(kTabThreads, 2)
     k_sample_tab(const __grid_constant__ View<float> V, int model, const double *E, long long n, uint32_t k0, uint32_t k1,
@@ -212,9 +216,9 @@ bool sample_from_shared(const View<float> &V, int model, int method, const doubl
   if (method != 0 || n < kTabMin) return false;
   const size_t bytes = sizeof(AliasBin<float>) * V.meta[model].nE * kNB;
   int device = 0, sms = 0;
-  if (bytes > 100 * 1024 || cudaGetDevice(&device) != cudaSuccess ||
+  if (bytes > kTabBytes || cudaGetDevice(&device) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-      cudaFuncSetAttribute(k_sample_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)) != cudaSuccess) {
+      cudaFuncSetAttribute(k_sample_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTabBytes)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -2,6 +2,7 @@
 memory.  A context made later, or a call on another thread, that needs less of
 it must leave room for those that need more."""
 import dataclasses
+import threading
 
 import pytest
 
@@ -45,3 +46,39 @@ def test_small_context_leaves_a_large_one_its_shared_memory(gvmod, kw):
     small.close()
     assert r["status"] == 0
     assert [r["counters"][k] for k in gvmod.COUNTER_NAMES[:11]] == [ref["counters"][k] for k in gvmod.COUNTER_NAMES[:11]]
+
+
+def test_two_threads_sample_different_models(gvmod):
+    """The tables of different models have different sizes (Compton 74 KB,
+    pairs 49 KB): two threads that sample one each get the samples that each
+    gets alone."""
+    import torch
+    ctx = gvmod.Context(W.pbps_electrons(1), gvmod.gv_default_config(stack_capacity=1 << 12))
+    n = 1 << 20
+    energy = torch.linspace(2.0, 1e4, n, dtype=torch.float64, device="cuda")
+    alone, errors = {}, []
+    for model in (0, 1):
+        alone[model] = torch.zeros((n, 3), dtype=torch.float64, device="cuda")
+        ctx.gv_unit_sample(model, 0, energy, 99, alone[model])
+    torch.cuda.synchronize()
+
+    def sample(model):
+        stream = torch.cuda.Stream()
+        out = torch.zeros((n, 3), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        try:
+            for _ in range(3000):
+                ctx.gv_unit_sample(model, 0, energy, 99, out, stream)
+        except gvmod.GvError as e:
+            errors.append(str(e))
+        stream.synchronize()
+        if not torch.equal(out, alone[model]):
+            errors.append(f"model {model}: other samples")
+
+    threads = [threading.Thread(target=sample, args=(m,)) for m in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    ctx.close()
+    assert not errors, errors
