@@ -2260,10 +2260,11 @@ template <typename R> class StateSlot {
         ev_(device >= 0 && device < kMaxDevices ? g_slot_free[sizeof(R) == 8 ? 1 : 0][device] : nullptr) {}
   StateSlot(const StateSlot &) = delete;
   StateSlot &operator=(const StateSlot &) = delete;
+  // wait for the previous user
+  cudaError_t wait() { return ev_ ? cudaStreamWaitEvent(st_, ev_, 0) : cudaErrorInvalidResourceHandle; }
   // wait for the previous user, then copy the record into the slot
   cudaError_t take(const DevState<R> *record) {
-    if (!ev_) return cudaErrorInvalidResourceHandle;
-    const cudaError_t e = cudaStreamWaitEvent(st_, ev_, 0);
+    const cudaError_t e = wait();
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(R) == 8)
       return cudaMemcpyToSymbolAsync(c_state_d, record, sizeof(DevState<R>), 0, cudaMemcpyDeviceToDevice, st_);
@@ -3065,11 +3066,6 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
       occ < 1)
     return GV_ERR_CUDA;
   const int grid = c->sm_count * std::min(occ, c->cfg.blocks_per_sm);
-  // the tallies and the event counts start from zero on every call
-  if (cudaMemsetAsync(edep, 0, sizeof(double) * n_events * c->nsub, st) != cudaSuccess ||
-      cudaMemsetAsync(escape_E, 0, sizeof(double) * n_events, st) != cudaSuccess ||
-      cudaMemsetAsync(base + kStaticEvliveOff, 0, sizeof(unsigned) * n_events, st) != cudaSuccess)
-    return GV_ERR_CUDA;
   DevState<float> s = make_state<float>(c);
   s.qmem = base + kStaticQueueOff;
   s.q_bytes = TrackLayout<float>::queue_bytes(kStaticCap);
@@ -3099,7 +3095,15 @@ extern "C" int gv_transport_static(void *ctx, const gv_primary *prim, long long 
   s.seed_lo = static_cast<unsigned>(seed);
   s.seed_hi = static_cast<unsigned>(seed >> 32);
   DevState<float> *S = reinterpret_cast<DevState<float> *>(base + kStaticStateOff);
-  StateSlot<float> slot(c->device, st);  // held until the last generation is queued
+  // Held until the call returns.  The scratch array is touched only from here
+  // on: a call of another thread may use it until then, and clearing its event
+  // counts would keep its in-flight cap from ever admitting the next event.
+  StateSlot<float> slot(c->device, st);
+  // the tallies and the event counts start from zero on every call
+  if (slot.wait() != cudaSuccess || cudaMemsetAsync(edep, 0, sizeof(double) * n_events * c->nsub, st) != cudaSuccess ||
+      cudaMemsetAsync(escape_E, 0, sizeof(double) * n_events, st) != cudaSuccess ||
+      cudaMemsetAsync(base + kStaticEvliveOff, 0, sizeof(unsigned) * n_events, st) != cudaSuccess)
+    return GV_ERR_CUDA;
   static_state_kernel<<<1, 1, 0, st>>>(s, S);
   if (slot.take(S) != cudaSuccess) return GV_ERR_CUDA;
   if (n > 0)
