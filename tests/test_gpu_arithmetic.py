@@ -111,3 +111,9 @@ def run(tmp_path_factory):
 def test_widening_is_exact_on_every_float(run):
     bad, which, _ = run(0)
     assert bad == 0, (bad, hex(which))
+
+
+def test_div_rn_is_the_ieee_quotient(run):
+    bad, which, checked = run(1, 1 << 28)
+    assert checked > 1 << 26
+    assert bad == 0, (bad, hex(which))
