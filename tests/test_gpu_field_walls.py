@@ -1,7 +1,8 @@
 """A step in a magnetic field that ends on a lateral wall: the wall is the one
 the pre-step direction points at, also where the field turns the track away
 from it within the step.  Positrons just above the tracking cut graze a wall
-and stop on it, so the two photons of their annihilation start there."""
+and stop on it, so the two photons of their annihilation start there.  And the
+field's own step limit, down to curvatures below the FP32 normal range."""
 import dataclasses
 import os
 
@@ -59,3 +60,34 @@ def test_track_turned_away_stops_on_its_wall(oracle_mod, axis, prec, sort):
     tol = 1e-9 if prec else 1e-4
     assert np.abs(r["edep"][same] - ref["edep"][same]).max() < tol
     assert np.abs(r["escape"][same] - ref["escape"][same]).max() < tol
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("tesla", [4.0, 1e-12, 1e-36, 1e-38, 1e-39, 1e-40])
+def test_step_limit_of_the_weakest_fields(oracle_mod, prec, tesla):
+    """The limit is the square root of a quotient by the curvature: finite
+    where that quotient is, although the curvature's reciprocal is not.  A
+    curvature below 1.2e-38 / cm holds multiples of 2^-149; it is rounded
+    three times on the way (constant, quotient by p, sine)."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    wl = W.with_field(W.pbps_electrons(1), tesla, 1)
+    ctx = gv.Context(wl, gv.gv_default_config(precision=prec, stack_capacity=1 << 12))
+    o = oracle_mod.Oracle(wl)
+    E = np.array([0.1, 1.0, 10.0, 30.0])
+    d = np.tile([[0.6, 0.0, 0.8]], (4, 1))
+    dev = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")
+    out = torch.zeros((4, 7), dtype=torch.float64, device="cuda")
+    ctx.gv_unit_field(1, dev(E), dev(np.full(4, 0.1)), dev(d), out)
+    got = out.cpu().numpy()[:, 6]
+    ctx.close()
+    for i in range(4):
+        want = o.field_step_limit(1, E[i], d[i])
+        curv = 2.99792458 * tesla / np.sqrt(E[i] * (E[i] + 2 * 0.51099895))
+        tol = 1e-5 + 3 * 2.0 ** -149 / curv if prec == 0 else 1e-12
+        if prec == 0 and want ** 2 > 3.4028235e38:  # the quotient overflows, as a division's does
+            assert got[i] == np.inf
+            continue
+        assert abs(got[i] - want) <= tol * want, (E[i], got[i], want)
