@@ -105,8 +105,7 @@ __global__ void k_distance(View<R> V, const double *pos, const double *dir, cons
     return;
   }
   const R d = distance(V, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], static_cast<R>(dir[3 * i]),
-                       static_cast<R>(dir[3 * i + 1]), static_cast<R>(dir[3 * i + 2]), sub[i],
-                       lateral_free(V.geo, pos[3 * i], pos[3 * i + 1]), nx, pl);
+                       static_cast<R>(dir[3 * i + 1]), static_cast<R>(dir[3 * i + 2]), sub[i], nx, pl);
   dist[i] = d;
   next[i] = nx;
   plane[i] = pl;
