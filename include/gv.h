@@ -319,7 +319,11 @@ long long gv_last_launches(void *ctx);
 
 /* ---- element-wise entry points (device pointers, asynchronous on stream) ----
  * They run the same device functions as gv_transport, in the context's
- * precision, one element per thread; inputs and outputs are FP64 arrays. */
+ * precision, one element per thread; inputs and outputs are FP64 arrays.  (The
+ * transport's runs of steps put the navigator's functions together themselves,
+ * and its final states, which gv_unit_interact runs, form a sampled model's
+ * physical variable from the reduced one in place; gv_unit_alias_sample and
+ * gv_unit_sample do that in a function of their own.) */
 
 /* Philox4x32-10 (Random123 family, Sec. 3.3.2): out[4i..4i+3] from counter
  * ctr[4i..4i+3] and key key[2i..2i+1]. */

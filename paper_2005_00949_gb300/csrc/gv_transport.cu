@@ -224,11 +224,11 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
   int gi;
   R gf;
   const R INF = r_inf<R>();
-  const bool up = t.w > R(0), plane_ahead = t.w != R(0);
+  const bool up = t.w > R(0);
   int sub = t.sub;
   GV_CHECK(&S->ctl->status, sub >= 0 && sub < geo.nsub);
   SubRec<R> rec = V.rec[sub];
-  R h = static_cast<R>(V.zb[up ? sub + 1 : sub] - t.z);
+  R h = static_cast<R>(V.zb[plane_ahead(t.w, sub)] - t.z);
   grid_pos_on(V.inv_node, t.E, gi, gf);
   GV_CHECK(&S->ctl->status, gi >= 0 && gi <= kGridN - 2);
   const V4<R> *const tab = V.xs + gi;
@@ -238,7 +238,7 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
   V4<R> sig = lerp4(tab[rec.row], tab[rec.row + 1], gf);  // ComputeIntLen
   R nlam = t.nlam, s;
   // GeomQuery
-  R d = plane_ahead ? by_w.div(h) : INF;
+  R d = way_to_plane(by_w, t.w, h);
   int m = 0, pl = -1;
   if (sizeof(R) == 4) {
     if (!walls_clear(lat, d)) walls(geo, t.x, t.y, t.u, t.v, d, d, pl);
@@ -267,12 +267,7 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
     s = s_phys < s ? s_phys : s;
     if (sizeof(R) == 8 && !walls_clear(lat, s)) {
       lat = lateral_free(geo, t.x, t.y);
-      R near = ahead;
-      walls(geo, t.x, t.y, t.u, t.v, s, near, pl);
-      if (pl < -1) {
-        d = near < R(0) ? R(0) : near;
-        s = d < s ? d : s;
-      }
+      if (nearer_wall(geo, t.x, t.y, t.u, t.v, s, ahead, d, pl)) s = d < s ? d : s;
     }
     finite = s < INF;
     geom = d == s;
@@ -354,14 +349,14 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
   double *const edep = S->edep + static_cast<size_t>(t.ev) * geo.nsub;
   GV_CHECK(&S->ctl->status, t.sub >= 0 && t.sub < geo.nsub);
   float lat = lateral_free(geo, t.x, t.y);
-  int plane = t.w > R(0) ? t.sub + 1 : t.sub;
+  int plane = plane_ahead(t.w, t.sub);
   R dz = static_cast<R>(T.zb[plane] - t.z);
   int row = T.rec[t.sub].row + (pos ? 2 * kGridN : kGridN);
   Divisor<R> by_w(t.w);
   int lim, wall = -1;
   // the first step's geometry; later ones start the plane's FP64 difference as
   // soon as z is known, and it is done when the loss is
-  R s_geom = t.w != R(0) ? by_w.div(dz) : INF;
+  R s_geom = way_to_plane(by_w, t.w, dz);
   int m = 0, end = kRunOn;
   for (;;) {
     ++r.n_iter;
@@ -404,17 +399,14 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     s = s_phys < s ? s_phys : s;
     if (!walls_clear(lat, s)) {
       lat = lateral_free(geo, t.x, t.y);
-      R near = ahead;
-      walls(geo, t.x, t.y, t.u, t.v, s, near, wall);
-      if (wall < -1) {
-        s_geom = near < R(0) ? R(0) : near;
+      if (nearer_wall(geo, t.x, t.y, t.u, t.v, s, ahead, s_geom, wall)) {
         s = s_geom < s ? s_geom : s;
         // the wall that the pre-step direction points at (-4, -5: the lower one):
         // a field may turn the track within the step
         if (!((wall == -2 ? t.u : t.v) > R(0))) wall -= 2;
       }
     }
-    const int next = wall < -1 ? -1 : (t.w > R(0) ? (t.sub + 1 < geo.nsub ? t.sub + 1 : -1) : t.sub - 1);
+    const int next = slab_behind(t.w, t.sub, geo.nsub, wall);
     lim = (s_geom == s) ? 0 : (s_phys == s ? 1 : 2);
     if (!(s < INF)) {
       escape<R, EXT>(S, t, -1, r);
@@ -455,7 +447,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
     const int crossed = plane;  // chosen with the pre-step direction
     if (lim == 0 && wall == -1) t.z = T.zb[crossed];
     const int pre_sub = t.sub, sub = lim == 0 && next >= 0 ? next : t.sub;
-    plane = t.w > R(0) ? sub + 1 : sub;
+    plane = plane_ahead(t.w, sub);
     if (!msc) dz = static_cast<R>(T.zb[plane] - t.z);
     row = T.rec[sub].row + (pos ? 2 * kGridN : kGridN);
     lat = lat_after(lat, s);
@@ -491,7 +483,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       t.u = dm[0];
       t.v = dm[1];
       t.w = dm[2];
-      plane = t.w > R(0) ? sub + 1 : sub;
+      plane = plane_ahead(t.w, sub);
       dz = static_cast<R>(T.zb[plane] - t.z);
       by_w = Divisor<R>(t.w);
     }
@@ -506,7 +498,7 @@ __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *
       break;
     }
     if (m >= budget || !(t.nlam > R(0))) break;
-    s_geom = t.w != R(0) ? by_w.div(dz) : INF;
+    s_geom = way_to_plane(by_w, t.w, dz);
     wall = -1;
   }
   return end;
@@ -1124,7 +1116,6 @@ template <typename R> __device__ __forceinline__ void stage_tables(const DevStat
     sV.inv_node = idst;
     sV.smat = mdst;
     if (S->smax_bytes) sV.smax = reinterpret_cast<const R *>(smem + S->smax_off);
-    sV.rec = rdst;
   }
   __syncthreads();
 }
@@ -1906,7 +1897,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? GV_ALONG_MIN_BLOCKS : 2)
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) interact_kernel(const DevState<R> *__restrict__ S, int parity) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) interact_kernel(const DevState<R> *__restrict__ S, int parity) {
   __shared__ View<R> sV;
   __shared__ WarpCnt s_wc[8];
   __shared__ unsigned s_kend[kNReqKey], s_kn[kNReqKey];
@@ -2184,7 +2175,6 @@ template <typename R> View<R> make_view(const Ctx *c) {
   v.smat = c->d_smat;
   v.bins = reinterpret_cast<const AliasBin<R> *>(c->d_bins);
   v.smax = reinterpret_cast<const R *>(c->d_smax);
-  v.rec = nullptr;  // made by the step kernels
   v.status = nullptr;  // unit kernels: no status word
   for (int m = 0; m < kNModel; ++m) v.meta[m] = c->meta[m];
   v.geo.nsub = c->nsub;
