@@ -117,3 +117,10 @@ def test_div_rn_is_the_ieee_quotient(run):
     bad, which, checked = run(1, 1 << 28)
     assert checked > 1 << 26
     assert bad == 0, (bad, hex(which))
+
+
+@pytest.mark.parametrize("lo, hi", [(1, 252), (0, 0)], ids=["normal", "subnormal"])
+def test_divisor_is_the_approximate_division(run, lo, hi):
+    bad, which, checked = run(2, 1 << 26, lo, hi)
+    assert checked > 1 << 24
+    assert bad == 0, (bad, hex(which))
