@@ -177,7 +177,8 @@ __global__ void k_sample(View<R> V, int model, int method, const double *E, long
 // bytes a bin, 49 KB for pairs) in the shared memory of persistent blocks.
 // k_sample reads them through L1, whose 32 lookups per 32 random bins bound
 // it (ncu: L1 75 %, issue 61 %, DRAM 23 %); a random 16-byte read of shared
-// memory passes a warp in about 12 cycles.  4M pair samples: 44 -> 37 us.
+// memory passes a warp in about 12 cycles.  4M pair samples: 45 -> 35 us.
+// Sample i has the same bits from either kernel (tests/test_gpu_sampler_sizes.py).
 constexpr int kTabThreads = 1024;
 // Below this many samples a block's copy of the rows costs more than it saves:
 // 2^18 samples take 8.1 us this way and 7.6 us through L1, 2^19 10.1 and
