@@ -127,7 +127,7 @@ typedef struct {
 typedef struct {
   int precision;              /* GV_MIXED or GV_FP64 */
   int mode;                   /* GV_BATCHED or GV_ONE_EVENT_PER_LAUNCH */
-  int block_size;             /* threads per block: 64..512, multiple of 32 */
+  int block_size;             /* threads per block: 64..256 (the library's GV_MAX_BLOCK), multiple of 32 */
   int blocks_per_sm;          /* persistent blocks per SM */
   int steps_per_claim;        /* steps a thread takes on a claimed track per generation */
   int tail_steps_per_claim;   /* the same when fewer than tail_threshold tracks are live */
@@ -234,10 +234,14 @@ int gv_build_tables(void *ctx);
 
 /* Transport n primaries (host or device array) of n_events events with the
  * given seed (the stepping loop of Sec. 2.1.2 stages, stack of Sec. 2.1.2,
- * scoring of Sec. 3.8.1), until every track has ended, and copy the tallies
- * into res's buffers.  The work is ordered after what the caller queued on
+ * scoring of Sec. 3.8.1), until every track has ended, with the tallies in
+ * res's buffers.  The work is ordered after what the caller queued on
  * `stream` before the call, and `stream` waits for it: work the caller
- * queues on it later sees the tallies.  The call returns once the work is
+ * queues on it later sees the tallies.  Tally buffers in this GPU's memory
+ * (cudaMalloc and the like, 8-byte aligned) are cleared and accumulated into
+ * while the transport runs, from where `stream` has reached the call on; all
+ * others (host, managed, another GPU's) change only when the results are
+ * copied at its end.  The call returns once the work is
  * enqueued (config blocking = 0, the default); res->counters, status and
  * kernel_ms are filled by gv_sync, which also returns the status, and the
  * tally buffers hold the results once `stream` has reached that point.  With
@@ -278,7 +282,8 @@ int gv_transport_events(void *ctx, const gv_primary *p, long long n, long long f
  * array and clears what must start at zero.  Like gv_transport it takes the
  * GPU's constant-memory state record in turn with every other transport,
  * and holds it until it returns: calls from several threads, streams or
- * contexts run one after another and do not share the array's contents.  The call waits on the host between its launches, so it cannot
+ * contexts run one after another and do not share the array's contents.
+ * The call waits on the host between its launches, so it cannot
  * run on a stream that is being captured (GV_ERR_BAD_ARG) and must not run
  * while another stream of the device captures in global mode.
  *   prim      device array of n primaries;

@@ -1455,9 +1455,9 @@ template <> __device__ __forceinline__ const DevState<double> *tstate<double>() 
 // small, because a warp fetches what it runs once per claim anew: the same
 // kernel with 12 KB more of it lost 5 % on the small transports.  What a caller
 // waits for, before these and with them: 2000 x 10 GeV e- in Pb/polystyrene
-// 7.74 -> 3.83 ms, 1000 x 1 GeV 1.37 -> 0.69 ms, one 10 GeV shower 1.13 -> 0.57
-// ms, 300 x 10 GeV in FP64 13.0 -> 8.3 ms, 2000 x 100 GeV in W/Si with cells
-// 94.5 -> 51.4 ms.
+// 7.69 -> 3.80 ms, 1000 x 1 GeV 1.41 -> 0.70 ms, one 10 GeV shower 1.20 -> 0.59
+// ms, 300 x 10 GeV in FP64 13.3 -> 8.5 ms, 2000 x 100 GeV in W/Si with cells
+// 95.4 -> 52.3 ms.
 template <typename R, bool SORT, bool MERGE, bool FIELD, bool OPTS, bool EXT, bool ALT = !SORT>
 __global__ void GV_STEP_BOUNDS
     step_kernel(int parity) {
@@ -1603,9 +1603,8 @@ __global__ void GV_STEP_BOUNDS
       // and continuous-limited steps need no final state) until its track is
       // due a discrete interaction, ends, or has taken its type's budget of
       // steps (photons cross layers in runs of boundary-limited steps; charged
-      // tracks are stopped more often by their continuous-loss limit: measured
-      // best at 5 and 3 on the benchmark); the block then baskets the
-      // interactions.
+      // tracks are stopped more often by their continuous-loss limit); the
+      // block then baskets the interactions.
       uint32_t kstep;
       R u2 = R(0), u3 = R(0);
       Run<R> run;
@@ -2640,7 +2639,7 @@ int run_transport(Ctx *c, const gv_primary *p, long long n, long long first_even
     c->ev_cap = n_events;
   }
   // the automatic events-in-flight cap of a batched transport budgets every
-  // event by its own primaries (prim_cost_kernel, plan_next)
+  // event by its own primaries (start_kernel, plan_next)
   const bool cost_cap = c->cfg.max_events_in_flight < 0 && c->cfg.mode == GV_BATCHED && n > 0;
   if (cost_cap && static_cast<size_t>(n) + 1 > c->pcost_cap) {
     cudaFree(c->d_pcost);
@@ -2794,9 +2793,11 @@ int gv_default_config(gv_config *cfg) {
   if (!cfg) return GV_ERR_BAD_ARG;
   cfg->precision = GV_MIXED;
   cfg->mode = GV_BATCHED;
-  // measured on 2000 x 10 GeV e- in Pb/polystyrene (GB300): the basketizing
-  // kernel with block claims, 2 blocks of 256 per SM, up to 3 along-steps per
-  // basket round for electrons and positrons and 5 for photons, one round
+  // measured on 2000 x 10 GeV e- in Pb/polystyrene (GB300), the budgets on an
+  // earlier form of the kernels: the basketizing kernel with block claims, 2
+  // blocks of 256 per SM, up to 3 along-steps per basket round for electrons
+  // and positrons and 5 for photons (8 would take 3 % less time in mixed
+  // precision now, one 10 GeV shower 8 %, and 1.4 % more in FP64), one round
   // per claim
   cfg->block_size = 256;
   cfg->blocks_per_sm = 2;
