@@ -210,13 +210,14 @@ __device__ __forceinline__ void escape(const DevState<R> *S, const Trk<R> &t, in
 // A run is one chain of dependent instructions, so the loop has one exit, and
 // the next sub-slab's record and cross sections are fetched before the exit is
 // decided: 480 -> 176 cycles a step for a warp alone on its SM.
-// In FP32 a run also ends where a wall may be nearer than the next plane:
-// looking at the walls again in the loop halves the time of photons in a box
-// narrower than its sub-slabs (0.80 -> 0.36 ms for 1e5 of 1 MeV, half width
-// 0.5 mm), but costs every other photon a second path through the loop (2000 x
-// 10 GeV 3.78 -> 3.85 ms).  FP64 steps are long enough not to feel it (300 x 10
-// GeV 8.36 ms both ways), and pay for the rounds of one step (300 x 1 GeV in a
-// box of 1 cm 5.29 ms, 3.04 looking again).
+// A run also ends where a wall may be nearer than the next plane, by the bound
+// along its direction (lateral_way): before the last step of a flight that ends
+// on a wall.  (That step in the same run, in the loop or after it, cost 2000 x 10
+// GeV 1 to 2 %.)  With a bound
+// that did not know the direction nearly every step ended a run in a box about
+// as wide as its layers are thick: 300 x 1 GeV in FP64 in a box of 1 cm took
+// 5.67 ms (now 3.05), 1000 x 1 GeV in mixed precision 1.36 (0.70), 1e5 photons
+// of 1 MeV in a box of 1 mm 0.75 (0.33).
 template <typename R, bool EXT>
 __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r) {
   const Staged<R> V(S);
@@ -233,17 +234,15 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
   GV_CHECK(&S->ctl->status, gi >= 0 && gi <= kGridN - 2);
   const V4<R> *const tab = V.xs + gi;
   const Divisor<R> by_w(t.w);
-  float lat = lateral_free(geo, t.x, t.y);
+  float lat = lateral_way(geo, t.x, t.y, t.u, t.v);
   const int last = geo.nsub - 1, dir = up ? 1 : -1;
   V4<R> sig = lerp4(tab[rec.row], tab[rec.row + 1], gf);  // ComputeIntLen
   R nlam = t.nlam, s;
   // GeomQuery
   R d = way_to_plane(by_w, t.w, h);
   int m = 0, pl = -1;
-  if (sizeof(R) == 4) {
-    if (!walls_clear(lat, d)) walls(geo, t.x, t.y, t.u, t.v, d, d, pl);
-    if (d < R(0)) d = R(0);
-  }
+  if (!walls_clear(lat, d)) walls(geo, t.x, t.y, t.u, t.v, d, d, pl);
+  if (d < R(0)) d = R(0);
   int row = rec.row, back_row = -1;  // of this sub-slab and the one before: table row, cross sections, path across
   V4<R> back_sig = sig;
   R back_h = R(0), back_d = R(0);
@@ -261,14 +260,8 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
       nsig = lerp4(tab[nrec.row], tab[nrec.row + 1], gf);
       nd = by_w.div(nh);
     }
-    const R ahead = d;
-    if (sizeof(R) == 8 && d < R(0)) d = R(0);
     s = INF < d ? INF : d;
     s = s_phys < s ? s_phys : s;
-    if (sizeof(R) == 8 && !walls_clear(lat, s)) {
-      lat = lateral_free(geo, t.x, t.y);
-      if (nearer_wall(geo, t.x, t.y, t.u, t.v, s, ahead, d, pl)) s = d < s ? d : s;
-    }
     finite = s < INF;
     geom = d == s;
     out = pl < -1 || static_cast<unsigned>(next) > static_cast<unsigned>(last);
@@ -299,7 +292,7 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
       row = nrec.row;
       h = nh;
     }
-    if (sizeof(R) == 4 && !walls_clear(lat, nd)) break;
+    if (!walls_clear(lat, nd)) break;
     sub = next;
     d = nd;
     sig = nsig;
@@ -334,11 +327,12 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
 // a boundary, by the continuous loss (or the field) or, the last one, by
 // physics.  1600 (step within one node interval) and 2100 cycles (across
 // several) a step for a warp alone on its SM became 950 and 1215.
-// The walls are looked at where the bound does not clear the step itself: its
-// other limits are known by then, and mostly millimetres, where the plane ahead
-// of a slanted track is far.  A run that ended wherever the bound did not clear
-// that plane took one step a round beside a wall (1000 x 1 GeV in a box of 1 cm
-// 1.36 ms, now 1.29; in 40 cm 2000 x 10 GeV 3.82 -> 3.78, TestEm3 in 4 T 5.74 -> 5.70).
+// The walls are looked at where the bound (lateral_free: the direction may
+// change) does not clear the step itself: its other limits are known by then, and
+// mostly millimetres, where the plane ahead of a slanted track is far.  A run
+// that ended wherever the bound did not clear that plane took one step a round
+// beside a wall (5000 x 10 MeV e- in FP64 in a box of 0.4 mm 1.15 -> 0.80 ms; in 40 cm
+// 2000 x 10 GeV 3.82 -> 3.78).
 template <typename R, bool FIELD, bool OPTS, bool EXT>
 __device__ __forceinline__ int charged_run(const View<R> &V, const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r,
                                            Pending<R> *pd) {

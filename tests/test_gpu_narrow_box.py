@@ -1,6 +1,6 @@
-"""Boxes whose lateral walls are nearer than the planes ahead, where nearly
-every step looks at the walls: histories do not depend on how steps are cut
-into runs, and a charged track takes its whole budget of steps there, too."""
+"""Boxes whose lateral walls are nearer than the planes ahead, where a bound to
+the nearest wall clears hardly any step: histories do not depend on how steps
+are cut into runs, and tracks take their whole budget of steps there, too."""
 import dataclasses
 import os
 
@@ -79,3 +79,34 @@ def test_charged_runs_go_on_beside_a_wall(oracle_mod, prec, sort):
     longest = oracle_mod.Oracle(wl).transport(n_threads=4)["counts"][:, 0].max()
     assert 10 < longest <= 64
     assert gens[0] >= longest and gens[1] <= 2, gens
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("sort", [dict(), dict(pipeline=1)], ids=["sort", "split"])
+def test_photon_runs_go_on_beside_a_wall(prec, sort):
+    """Photons that do not interact, across 50 slabs of half a millimetre, 0.1 to
+    0.9 mm from the walls and slowly towards them: with one round a generation
+    and a budget of 64 steps they cross in one run.  Those that reach a wall
+    take the last step in a second one, or a third where the first ended a step
+    early: the bound is short by a thousandth of a step and 1e-4 of the path."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2005_00949_gb300 import gv
+    n = 64
+    wl = dataclasses.replace(_narrow(n), n_layers=50, sub_thick=[0.05], half_x=0.1, half_y=0.1, process_mask=W.P_PAIR)
+    p = wl.primaries
+    p["type"], p["E"] = W.GAMMA, 0.9
+    p["x"], p["y"] = np.linspace(0.01, 0.09, n), -np.linspace(0.09, 0.01, n)
+    p["u"], p["v"] = np.linspace(0.0, 0.03, n), -np.linspace(0.03, 0.0, n)
+    p["w"] = np.sqrt(1.0 - p["u"] ** 2 - p["v"] ** 2)
+    gens, escaped = [], []
+    for budget in (1, 64):
+        ctx = gv.Context(wl, gv.gv_default_config(precision=prec, stack_capacity=1 << 12, along_steps_photon=budget,
+                                                  tail_threshold=0, **sort))
+        r = ctx.transport()
+        ctx.close()
+        assert r["status"] == 0
+        gens.append(r["counters"]["generations"])
+        escaped.append((r["counters"]["steps"], r["counters"]["unscattered"], r["escape"].tolist()))
+    assert escaped[0] == escaped[1] and 0 < escaped[0][1] < n  # some leave through the far plane, some through a wall
+    assert gens[0] >= 50 and gens[1] <= 3, gens
