@@ -210,14 +210,13 @@ __device__ __forceinline__ void escape(const DevState<R> *S, const Trk<R> &t, in
 // A run is one chain of dependent instructions, so the loop has one exit, and
 // the next sub-slab's record and cross sections are fetched before the exit is
 // decided: 480 -> 176 cycles a step for a warp alone on its SM.
-// A run also ends where a wall may be nearer than the next plane, by the bound
-// along its direction (lateral_way): before the last step of a flight that ends
-// on a wall.  (That step in the same run, in the loop or after it, cost 2000 x 10
-// GeV 1 to 2 %.)  With a bound
-// that did not know the direction nearly every step ended a run in a box about
-// as wide as its layers are thick: 300 x 1 GeV in FP64 in a box of 1 cm took
-// 5.67 ms (now 3.05), 1000 x 1 GeV in mixed precision 1.36 (0.70), 1e5 photons
-// of 1 MeV in a box of 1 mm 0.75 (0.33).
+// A run also ends where a wall may limit the next step, by the bound along its
+// direction (lateral_way): before the last step of a flight that ends on a wall.
+// (That step in the same run, in the loop or after it, cost 2000 x 10 GeV 1 to
+// 2 %.)  With a bound that did not know the direction, against the next plane,
+// nearly every step ended a run in a box about as wide as its layers are thick:
+// 300 x 1 GeV in FP64 in a box of 1 cm took 5.67 ms (now 3.04), 1000 x 1 GeV in
+// mixed precision 1.36 (0.70), 1e5 photons of 1 MeV in a box of 1 mm 0.75 (0.33).
 template <typename R, bool EXT>
 __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int budget, Run<R> &r) {
   const Staged<R> V(S);
@@ -248,9 +247,11 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
   R back_h = R(0), back_d = R(0);
   h = R(0);  // (the first path starts inside)
   bool finite, geom, out;
+  R Sig = sig.x + sig.y + sig.z;
+  R s_phys = Sig > R(0) ? q_div(nlam, Sig) : INF;
+  s = INF < d ? INF : d;
+  s = s_phys < s ? s_phys : s;
   for (;;) {
-    const R Sig = sig.x + sig.y + sig.z;
-    const R s_phys = Sig > R(0) ? q_div(nlam, Sig) : INF;
     const int next = sub + dir;
     const SubRec<R> nrec = V.rec[min(max(next, 0), last)];
     const R nh = up ? nrec.thick : -nrec.thick;  // from the plane it enters through
@@ -260,8 +261,6 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
       nsig = lerp4(tab[nrec.row], tab[nrec.row + 1], gf);
       nd = by_w.div(nh);
     }
-    s = INF < d ? INF : d;
-    s = s_phys < s ? s_phys : s;
     finite = s < INF;
     geom = d == s;
     out = pl < -1 || static_cast<unsigned>(next) > static_cast<unsigned>(last);
@@ -292,7 +291,11 @@ __device__ __forceinline__ int photon_run(const DevState<R> *S, Trk<R> &t, int b
       row = nrec.row;
       h = nh;
     }
-    if (!walls_clear(lat, nd)) break;
+    Sig = nsig.x + nsig.y + nsig.z;
+    s_phys = Sig > R(0) ? q_div(nlam, Sig) : INF;
+    s = INF < nd ? INF : nd;
+    s = s_phys < s ? s_phys : s;
+    if (!walls_clear(lat, s)) break;
     sub = next;
     d = nd;
     sig = nsig;
